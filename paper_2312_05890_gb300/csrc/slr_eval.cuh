@@ -79,6 +79,44 @@ template <> __device__ __forceinline__ void lds4<double>(uint32_t addr, double (
     asm volatile("ld.shared.v2.f64 {%0, %1}, [%2+16];" : "=d"(v[2]), "=d"(v[3]) : "r"(addr));
 }
 
+// Two floats as one 64-bit register pair, for Blackwell's packed FP32
+// instructions (fma.rn.f32x2: two independent FMAs, each rounded as fmaf).
+// A packed FMA fills the FP32 pipe as two plain ones do, so it saves issue
+// slots only; the products, where the pipe itself is busy, gain little: a
+// 22-64-64-3 count of depth 18 9.68 -> 9.50 ms, 200,001 boxes of a 5-6x50-5
+// network 2.76 -> 2.71 ms, its depth-20 count 26.2 -> 25.9 ms (the float64
+// re-check's float-float products included).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// a - b in each half (-1 * b is exact, so the sum is rounded once)
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, 0xbf800000bf800000ull, a); }
+// Four consecutive floats as two pairs from a 32-bit shared address.
+__device__ __forceinline__ void lds2x2(uint32_t addr, f32x2 (&v)[2]) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(addr));
+}
+
 template <typename Real> struct V4;
 template <> struct V4<float> {
     static __device__ __forceinline__ void ld(const float *p, float (&v)[4]) {
@@ -223,15 +261,19 @@ __device__ __forceinline__ double ff_abs(double wabs, int n, int d) {
     return __dmul_ru((double)(2 * d + 8) * 0x1p-149, __dadd_ru(wabs, (double)(2 * n + 8)));
 }
 
-// Multiply-add of a float weight and a float-float input into a float-float
-// accumulator (s, e): the product exactly as p + pe, p added to s by TwoSum,
-// the error terms and w lo added to e in float.
-__device__ __forceinline__ void ff_mac(float w, float h, float l, float &s, float &e) {
-    float p, pe, t, se;
-    two_prod<float>(w, h, p, pe);
-    two_sum<float>(s, p, t, se);
+// Multiply-add of two float weights and one float-float input (h and l in both
+// halves, nh = -h) into float-float accumulators (s, e): the product exactly
+// as p + pe, p added to s by TwoSum, the error terms and w l added to e in
+// float (w (-h) is the product's negative, exactly).
+__device__ __forceinline__ void ff_mac2(f32x2 w, f32x2 h, f32x2 nh, f32x2 l, f32x2 &s, f32x2 &e) {
+    const f32x2 np = mul2(w, nh);            // -p
+    const f32x2 pe = fma2(w, h, np);         // the product's error
+    const f32x2 t = sub2(s, np);             // s + p
+    const f32x2 z = sub2(t, s);
+    const f32x2 a = sub2(s, sub2(t, z));
+    const f32x2 se = sub2(a, add2(np, z));   // a + (p - z)
     s = t;
-    e = __fmaf_rn(w, l, __fadd_rn(e, __fadd_rn(pe, se)));
+    e = fma2(w, l, add2(e, add2(pe, se)));
 }
 
 // Row accessors.  A row view R maps a column of one row (SIMT numbering: C
@@ -947,6 +989,35 @@ struct EvalTile {
         }
     }
 
+    template <bool kAbs>
+    static __device__ __forceinline__ void mac_rows2(uint32_t w0, uint32_t x0, const int2 *rows, int n_rows,
+                                                     f32x2 (&acc)[4][4]) {
+#pragma unroll 2
+        for (int ii = 0; ii < n_rows; ++ii) {
+            const int2 o = rows[ii];
+            f32x2 wa[2], wb[2];
+            float x[4];
+            lds2x2(w0 + (uint32_t)o.x, wa);
+            lds2x2(w0 + (uint32_t)o.x + 16u, wb);
+            lds4<float>(x0 + (uint32_t)o.y, x);
+            if (kAbs) {
+                constexpr f32x2 kMag = 0x7fffffff7fffffffull;
+                wa[0] &= kMag;
+                wa[1] &= kMag;
+                wb[0] &= kMag;
+                wb[1] &= kMag;
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const f32x2 xx = pack2(x[c], x[c]);
+                acc[0][c] = fma2(wa[0], xx, acc[0][c]);
+                acc[1][c] = fma2(wa[1], xx, acc[1][c]);
+                acc[2][c] = fma2(wb[0], xx, acc[2][c]);
+                acc[3][c] = fma2(wb[1], xx, acc[3][c]);
+            }
+        }
+    }
+
     // The same product over the rows of a list: rows[ii] = byte offsets (i Mpad,
     // i NS) of the rows i to sum over; a row that is zero in every box of the
     // tile adds exact zeros, so leaving it out changes no sum.
@@ -957,6 +1028,22 @@ struct EvalTile {
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[r][c] = 0;
         const uint32_t w0 = (uint32_t)__cvta_generic_to_shared(wp), x0 = (uint32_t)__cvta_generic_to_shared(xp);
+        if constexpr (sizeof(Real) == 4) {
+            // pairs of neighbouring rows: the weights come as pairs from
+            // shared memory, the input is repeated in both halves
+            f32x2 a2[4][4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) a2[r][c] = 0ull;
+            if (is_abs) mac_rows2<true>(w0, x0, rows, n_rows, a2);
+            else mac_rows2<false>(w0, x0, rows, n_rows, a2);
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) unpack2(a2[r][c], acc[2 * r][c], acc[2 * r + 1][c]);
+            return;
+        }
         if (is_abs) {
 #pragma unroll 2
             for (int ii = 0; ii < n_rows; ++ii) {
@@ -1135,7 +1222,7 @@ struct EvalTile {
     // instead: every input x of the state is split into float hi + lo
     // (x - hi is exact, lo = fl(x - hi): |x - hi - lo| <= 2^-48 |x| + 2^-150),
     // each term w hi is formed exactly, and the sums carry a float error term
-    // (ff_mac).  The result hi + lo, rounded to float64, is within
+    // (ff_mac2).  The result hi + lo, rounded to float64, is within
     // gam_ff(n) sum_i |w_i| |x_i| + ff_abs of the exact product: the
     // contraction's rounding bound that the next epilogue takes in place of
     // gamma_n.
@@ -1159,35 +1246,39 @@ struct EvalTile {
     static __device__ __forceinline__ void tile_mac_rows_ff(const float *wp, const float *xh, const float *xl,
                                                             const int *ridx, int n_rows, int Mpad, int NP,
                                                             bool is_abs, float (&sh)[8][4], float (&sl)[8][4]) {
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) sh[r][c] = sl[r][c] = 0.f;
         const uint32_t w0 = (uint32_t)__cvta_generic_to_shared(wp);
         const uint32_t h0 = (uint32_t)__cvta_generic_to_shared(xh), l0 = (uint32_t)__cvta_generic_to_shared(xl);
+        // pairs of neighbouring rows (see mac_rows2)
+        f32x2 s2[4][4], e2[4][4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) s2[r][c] = e2[r][c] = 0ull;
+        const f32x2 mag = is_abs ? 0x7fffffff7fffffffull : ~0ull;
         for (int ii = 0; ii < n_rows; ++ii) {
             const uint32_t i = (uint32_t)ridx[ii];
             const uint32_t ow = i * (uint32_t)(Mpad * 4), ox = i * (uint32_t)(NP * 4);
-            float a0[4], a1[4], h[4], l[4];
-            lds4<float>(w0 + ow, a0);
-            lds4<float>(w0 + ow + 16u, a1);
+            f32x2 wa[2], wb[2];
+            float h[4], l[4];
+            lds2x2(w0 + ow, wa);
+            lds2x2(w0 + ow + 16u, wb);
             lds4<float>(h0 + ox, h);
             lds4<float>(l0 + ox, l);
-            if (is_abs) {
+            const f32x2 w[4] = {wa[0] & mag, wa[1] & mag, wb[0] & mag, wb[1] & mag};
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    a0[r] = fabsf(a0[r]);
-                    a1[r] = fabsf(a1[r]);
-                }
+            for (int c = 0; c < 4; ++c) {
+                const f32x2 hh = pack2(h[c], h[c]), nh = pack2(-h[c], -h[c]), ll = pack2(l[c], l[c]);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) ff_mac2(w[r], hh, nh, ll, s2[r][c], e2[r][c]);
             }
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    ff_mac(a0[r], h[c], l[c], sh[r][c], sl[r][c]);
-                    ff_mac(a1[r], h[c], l[c], sh[r + 4][c], sl[r + 4][c]);
-                }
         }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                unpack2(s2[r][c], sh[2 * r][c], sh[2 * r + 1][c]);
+                unpack2(e2[r][c], sl[2 * r][c], sl[2 * r + 1][c]);
+            }
     }
 
     // hi + lo of a finished tile into the state, all but the constant column
