@@ -109,6 +109,8 @@ struct slr_ctx {
     int64_t H = 0;                        // hidden neurons (slope row length)
     int adj_nck = 0, adj_grid = 0, adj_nmax = 0, adj_boxes = 1;
     bool adj_gmem = false;                // adjoint state in global memory (wide networks)
+    slr::AdjWarpPlan adjw{};              // one warp per box, where the network fits (tile path)
+    bool adjw_stale = true;               // planned at the first adjoint of a network
     void *adj_scratch = nullptr;
     size_t adj_scratch_bytes = 0;
     size_t adj_smem = 0;
@@ -857,6 +859,11 @@ int run_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int grid, int64_t *launches
     bool weights = false;
     for (int k = 0; k < ctx->nf.K; ++k) weights = weights || a.dW[k] != nullptr || a.db[k] != nullptr;
     if (ctx->wide && ctx->nf.K > 1 && !weights) return run_wide_adjoint(ctx, a, launches);
+    if (ctx->adjw.grid[weights] > 0) {
+        CK(ctx, slr::launch_adj_warp(a, ctx->adjw, weights, (float *)ctx->adj_scratch, ctx->stream));
+        *launches += 1;
+        return SLR_OK;
+    }
     CK(ctx, slr::launch_adjoint(a, grid, ctx->stream));
     *launches += 1;
     return SLR_OK;
@@ -936,6 +943,7 @@ void choose_recheck_tile(slr_ctx *ctx) {
 
 int prepare_device(slr_ctx *ctx) {
     if (!ctx->dev_dirty) return SLR_OK;
+    ctx->adjw_stale = true;
     if (ctx->widths.back() != (int)(ctx->C.size() / std::max<size_t>(1, ctx->e.size())))
         return fail(ctx, SLR_EINVAL, "property has %zu outputs per row but the network has %d outputs",
                     ctx->C.size() / std::max<size_t>(1, ctx->e.size()), ctx->widths.back());
@@ -2952,16 +2960,21 @@ int check_adjoint(slr_ctx *ctx) {
     if (ctx->adj_grid <= 0)
         return fail(ctx, SLR_EUNSUPPORTED, "network too large for the adjoint kernel (%zu bytes of shared memory)",
                     ctx->adj_smem);
-    if (ctx->adj_gmem) {
-        slr::AdjArgs a = adj_base(ctx);
-        const size_t need = slr::adjoint_box_bytes(a) * (size_t)ctx->adj_grid;
-        if (ctx->adj_scratch_bytes < need) {
-            cudaFree(ctx->adj_scratch);
-            ctx->adj_scratch = nullptr;
-            ctx->adj_scratch_bytes = 0;
-            CK(ctx, cudaMalloc(&ctx->adj_scratch, need));
-            ctx->adj_scratch_bytes = need;
-        }
+    if (ctx->adjw_stale) {
+        ctx->adjw = slr::AdjWarpPlan{};
+        if (!ctx->wide) slr::adj_warp_plan(ctx->nf, ctx->sm_count, (size_t)kMaxSmem, ctx->adjw);
+        ctx->adjw_stale = false;
+    }
+    size_t need = 0;
+    if (ctx->adj_gmem) need = slr::adjoint_box_bytes(adj_base(ctx)) * (size_t)ctx->adj_grid;
+    for (int w = 0; w < 2; ++w)
+        if (ctx->adjw.grid[w] > 0) need = std::max(need, slr::adj_warp_scratch_bytes(ctx->adjw, ctx->K, w != 0));
+    if (ctx->adj_scratch_bytes < need) {
+        cudaFree(ctx->adj_scratch);
+        ctx->adj_scratch = nullptr;
+        ctx->adj_scratch_bytes = 0;
+        CK(ctx, cudaMalloc(&ctx->adj_scratch, need));
+        ctx->adj_scratch_bytes = need;
     }
     return SLR_OK;
 }

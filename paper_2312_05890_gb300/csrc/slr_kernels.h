@@ -106,6 +106,20 @@ size_t adjoint_smem_bytes(const AdjArgs &a);
 size_t adjoint_box_bytes(const AdjArgs &a);
 int adjoint_blocks_per_sm(size_t smem);
 cudaError_t launch_adjoint(const AdjArgs &a, int grid, cudaStream_t s);
+// The same adjoint with one warp per box, for networks of at most 7 inputs and
+// layers at most 128 wide (slr_adj_warp.cu).  Index 0 of threads, grid and box:
+// without weight gradients, 1: with.
+struct AdjWarpPlan {
+    int QP, RPL;                    // columns of a row (d + 1 padded), rows a lane holds
+    int head;                       // floats of the staged weights and biases
+    int rows;                       // floats of one box's rows (widest layer x 2 QP)
+    int box[2];                     // floats of one warp's shared memory
+    int threads[2], grid[2];        // block size, largest grid (0: the network does not fit)
+    int w_off[kMaxLayers], w_ld[kMaxLayers], b_off[kMaxLayers];
+};
+void adj_warp_plan(const NetParams<float> &net, int sms, size_t smem_max, AdjWarpPlan &p);
+size_t adj_warp_scratch_bytes(const AdjWarpPlan &p, int K, bool weights);
+cudaError_t launch_adj_warp(const AdjArgs &a, const AdjWarpPlan &p, bool weights, float *chk, cudaStream_t s);
 // The adjoint on the wide path (per-layer tensor-core products; slr_wide_adj.cu).
 cudaError_t launch_wadj_box(const BoxSource &src, int64_t pos0, int nb, int d, float *m, float *r, int sms,
                             cudaStream_t s);
