@@ -123,6 +123,9 @@ struct slr_ctx {
     const float *w_hi[slr::kMaxLayers] = {}, *w_lo[slr::kMaxLayers] = {};
     const float *wa_hi[slr::kMaxLayers] = {}, *wa_lo[slr::kMaxLayers] = {};
     const float *w0t = nullptr;           // layer 1 transposed (d x n_1)
+    bool wide_layers = false;             // hidden layers by wide_layer_kernel
+    const float *w0p = nullptr;           // layer 1 transposed, rows padded with zeros (d x wide_NP)
+    const unsigned char *w_img[slr::kMaxLayers] = {};   // its weight pieces per layer
     int w_Kpad[slr::kMaxLayers] = {};
     // transposed pieces (W_k^T, |W_k|^T) for the adjoint's backward products
     const float *wt_hi[slr::kMaxLayers] = {}, *wt_lo[slr::kMaxLayers] = {};
@@ -568,6 +571,11 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
     ctx->wide_NP = np;
     std::vector<size_t> offs(K, 0), offs_t(K, 0);
     size_t total = align_up((size_t)d * nf.n[1] * sizeof(float));   // W_1 transposed first
+    // one kernel per hidden layer where its column tiles of one box are filled
+    // by at least kWideLayerMinD inputs and the property's rows fit its product
+    ctx->wide_layers = K > 1 && nf.R <= 16 && d >= slr::kWideLayerMinD;
+    const size_t off_w0p = total;
+    if (ctx->wide_layers) total += align_up((size_t)d * np * sizeof(float));
     for (int k = 1; k < K; ++k) {
         const int Mpad = (nf.n[k + 1] + 127) & ~127, Kpad = (nf.n[k] + 31) & ~31;
         ctx->w_Kpad[k] = Kpad;
@@ -578,13 +586,25 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
         offs_t[k] = total;
         total += 4 * align_up((size_t)MpadT * KpadT * sizeof(float));
     }
+    // (packed on the device from the pieces uploaded below)
+    const size_t host_total = total;
+    std::vector<size_t> offs_l(K, 0);
+    for (int k = 1; k + 1 < K && ctx->wide_layers; ++k) {
+        offs_l[k] = total;
+        total += align_up(slr::wide_layer_img_bytes(nf.n[k], nf.n[k + 1]));
+    }
     if (ctx->wide_img) cudaFree(ctx->wide_img);
     ctx->wide_img = nullptr;
     {
-        std::vector<unsigned char> host(total, 0);
+        std::vector<unsigned char> host(host_total, 0);
         float *w0t = (float *)host.data();
         for (int p = 0; p < nf.n[1]; ++p)
             for (int j = 0; j < d; ++j) w0t[(size_t)j * nf.n[1] + p] = L.W[0][(size_t)p * d + j];
+        if (ctx->wide_layers) {
+            float *w0p = (float *)(host.data() + off_w0p);
+            for (int j = 0; j < d; ++j)
+                std::memcpy(w0p + (size_t)j * np, w0t + (size_t)j * nf.n[1], nf.n[1] * sizeof(float));
+        }
         for (int k = 1; k < K; ++k) {
             const int n_in = nf.n[k], n_out = nf.n[k + 1];
             const int Mpad = (n_out + 127) & ~127, Kpad = ctx->w_Kpad[k];
@@ -618,9 +638,10 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
             }
         }
         CK(ctx, cudaMalloc(&ctx->wide_img, total));
-        CK(ctx, cudaMemcpy(ctx->wide_img, host.data(), total, cudaMemcpyHostToDevice));
-        ctx->h2d_pending += (int64_t)total;
+        CK(ctx, cudaMemcpy(ctx->wide_img, host.data(), host_total, cudaMemcpyHostToDevice));
+        ctx->h2d_pending += (int64_t)host_total;
         ctx->w0t = (const float *)ctx->wide_img;
+        ctx->w0p = (const float *)((const unsigned char *)ctx->wide_img + off_w0p);
         for (int k = 1; k < K; ++k) {
             const int Mpad = (nf.n[k + 1] + 127) & ~127;
             const size_t one = align_up((size_t)Mpad * ctx->w_Kpad[k] * sizeof(float));
@@ -635,6 +656,12 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
             ctx->wt_lo[k] = (const float *)(bt + oneT);
             ctx->wta_hi[k] = (const float *)(bt + 2 * oneT);
             ctx->wta_lo[k] = (const float *)(bt + 3 * oneT);
+            if (k + 1 < K && ctx->wide_layers) {
+                unsigned char *img = (unsigned char *)ctx->wide_img + offs_l[k];
+                CK(ctx, slr::launch_wide_pack(ctx->w_hi[k], ctx->w_lo[k], ctx->wa_hi[k], ctx->wa_lo[k],
+                                              ctx->w_Kpad[k], nf.n[k], nf.n[k + 1], img, ctx->stream));
+                ctx->w_img[k] = img;
+            }
         }
     }
     // chunk: the boxes whose state fits about 3 GB
@@ -651,8 +678,13 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
 int ensure_wide_buf(slr_ctx *ctx) {
     const int d = ctx->nf.d, np = ctx->wide_NP, R = ctx->nf.R;
     const size_t bc = (size_t)ctx->wide_Bc;
-    const size_t need = 2 * align_up(bc * d * np * 4) + 2 * align_up(bc * (d + 3) * np * 4) + 5 * align_up(bc * np * 4) +
-                        3 * align_up(bc * d * 4) + 3 * align_up(bc * R * 4) + align_up(bc * 8);
+    size_t need = 2 * align_up(bc * d * np * 4) + 2 * align_up(bc * (d + 3) * np * 4) + 5 * align_up(bc * np * 4) +
+                  3 * align_up(bc * d * 4) + 3 * align_up(bc * R * 4) + align_up(bc * 8);
+    if (ctx->wide_layers) {
+        int ntile, nc;
+        slr::wide_layer_tiles(d, ntile, nc);
+        need += align_up(bc * 2 * np * 4) + 2 * align_up(bc * 3 * np * 4) + align_up(bc * 8 * ntile * np * 4);
+    }
     if (ctx->wide_buf_bytes >= need) return SLR_OK;
     cudaFree(ctx->wide_buf);
     ctx->wide_buf = nullptr;
@@ -683,10 +715,86 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
     float *mh = take(bc * d * 4), *ml = take(bc * d * 4), *rr = take(bc * d * 4);
     float *lo = take(bc * R * 4), *hi = take(bc * R * 4), *er = take(bc * R * 4);
     int64_t *bidx = (int64_t *)take(bc * 8);
+    float *plan = nullptr, *S3 = nullptr, *T3 = nullptr, *part = nullptr;
+    if (ctx->wide_layers) {
+        plan = take(bc * 2 * np * 4);
+        S3 = take(bc * 3 * np * 4);
+        T3 = take(bc * 3 * np * 4);
+        part = (float *)p;
+    }
+    const bool prof = ctx->opt.profile != 0;
+    // an event before (0) and after (1) each tensor-core product when profiling
+    auto mark = [&](int after) -> cudaError_t {
+        if (!prof) return cudaSuccess;
+        while (ctx->gemm_ev.size() < ctx->gemm_ev_used + 2) {
+            cudaEvent_t e;
+            const cudaError_t ce = cudaEventCreate(&e);
+            if (ce != cudaSuccess) return ce;
+            ctx->gemm_ev.push_back(e);
+        }
+        const cudaError_t re = cudaEventRecord(ctx->gemm_ev[ctx->gemm_ev_used + after], ctx->stream);
+        if (after) ctx->gemm_ev_used += 2;
+        return re;
+    };
     for (int64_t base = 0; base < n; base += (int64_t)bc) {
         const int nb = (int)std::min<int64_t>((int64_t)bc, n - base);
         CK(ctx, slr::launch_wide_box(src, base, nb, d, mh, ml, rr, bidx, sms, ctx->stream));
         int cur = 0;
+        if (ctx->wide_layers) {
+            CK(ctx, slr::launch_wide_plan1(nf, ctx->w0p, nb, np, mh, ml, rr, plan, S3, Ch, Cl, src.alpha, src.alpha_ld,
+                                           base, ctx->stream));
+            *launches += 2;
+            for (int k = 1; k + 1 < K; ++k) {
+                const int nxt = cur ^ 1;
+                slr::WideLayer g{};
+                g.Aimg = ctx->w_img[k];
+                g.Cin = k > 1 ? Cb[cur] : nullptr;
+                g.Rin = k > 1 ? Rb[cur] : nullptr;
+                g.W0p = ctx->w0p;
+                g.rr = rr;
+                g.plan = plan;
+                g.Cout = Cb[nxt];
+                g.Rout = Rb[nxt];
+                g.part = part;
+                g.nb = nb;
+                g.d = d;
+                g.NP = np;
+                g.n_in = nf.n[k];
+                g.n_out = nf.n[k + 1];
+                g.status = out.status;
+                CK(ctx, mark(0));
+                CK(ctx, slr::launch_wide_layer(g, sms, ctx->stream));
+                // the radius constant, N and E columns
+                slr::WideGemmArgs ga{};
+                ga.status = out.status;
+                ga.g[0] = slr::WideGemm{ctx->wa_hi[k], ctx->wa_lo[k], S3, T3, nf.n[k + 1], nf.n[k], ctx->w_Kpad[k],
+                                        3 * nb, np, np};
+                CK(ctx, slr::launch_wide_gemm(ga, 1, ctx->stream));
+                CK(ctx, mark(1));
+                ctx->gemm_launches += 1;
+                ctx->gemm_flop += 2.0 * nf.n[k + 1] * nf.n[k] * ((double)nb * (2 * d + 1));
+                CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, S3 + np, 3 * (int64_t)np, Kh, Kl, Ke, sms,
+                                               ctx->stream));
+                CK(ctx, slr::launch_wide_plan(nf, k + 1, nb, np, slr::tc_gamma(ctx->w_Kpad[k]), part, T3, Kh, Kl, Ke,
+                                              plan, S3, Ch, Cl, src.alpha, src.alpha_ld, base, ctx->stream));
+                *launches += 4;
+                cur = nxt;
+            }
+            // the property layer: a few rows, on the CUDA cores
+            const bool gen = K == 2;
+            float *cols = Cb[cur ^ 1];
+            CK(ctx, slr::launch_wide_rows(nf, nb, np, gen ? nullptr : Cb[cur], gen ? nullptr : Rb[cur], ctx->w0p, rr,
+                                          plan, cols, sms, ctx->stream));
+            CK(ctx, slr::launch_wide_rows_product(nf.Wt[K - 1], nf.n[K - 1], R, S3, np, T3, np, 3 * (int64_t)nb, true,
+                                                  sms, ctx->stream));
+            CK(ctx, slr::launch_wide_const(nf, K - 1, nb, np, Ch, Cl, S3 + np, 3 * (int64_t)np, Kh, Kl, Ke, sms,
+                                           ctx->stream));
+            CK(ctx, slr::launch_wide_rows_final(nf, nb, np, (float)(nf.n[K - 1] + 2) * 0x1p-24f, cols, T3, Kh, Kl, Ke,
+                                                lo, hi, er, ctx->stream));
+            CK(ctx, slr::launch_wide_classify(nf, nb, base, lo, hi, er, bidx, out, sms, ctx->stream));
+            *launches += 5;
+            continue;
+        }
         CK(ctx, slr::launch_wide_init(nf, ctx->w0t, nb, np, mh, ml, rr, Cb[cur], Rb[cur], Ch, Cl, src.alpha,
                                       src.alpha_ld, base, ctx->stream));
         *launches += 2;
@@ -699,7 +807,8 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
                                                       (int64_t)nb * d, false, sms, ctx->stream));
                 CK(ctx, slr::launch_wide_rows_product(nf.Wt[k], nf.n[k], nf.R, Rb[cur], np, Rb[nxt], np,
                                                       (int64_t)nb * (d + 3), true, sms, ctx->stream));
-                CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur], Kh, Kl, Ke, sms, ctx->stream));
+                CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur] + (size_t)(d + 1) * np, (int64_t)(d + 3) * np,
+                                           Kh, Kl, Ke, sms, ctx->stream));
                 const float gf = (float)(nf.n[k] + 2) * 0x1p-24f;
                 CK(ctx, slr::launch_wide_final(nf, nb, np, gf, Cb[nxt], Rb[nxt], Ch, Cl, Kh, Kl, Ke, lo, hi, er,
                                                ctx->stream));
@@ -713,23 +822,13 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
                                     nb * d, np, np};
             ga.g[1] = slr::WideGemm{ctx->wa_hi[k], ctx->wa_lo[k], Rb[cur], Rb[nxt], nf.n[k + 1], nf.n[k],
                                     ctx->w_Kpad[k], nb * (d + 3), np, np};
-            const bool prof = ctx->opt.profile != 0;
-            if (prof) {
-                while (ctx->gemm_ev.size() < ctx->gemm_ev_used + 2) {
-                    cudaEvent_t e;
-                    CK(ctx, cudaEventCreate(&e));
-                    ctx->gemm_ev.push_back(e);
-                }
-                CK(ctx, cudaEventRecord(ctx->gemm_ev[ctx->gemm_ev_used], ctx->stream));
-            }
+            CK(ctx, mark(0));
             CK(ctx, slr::launch_wide_gemm(ga, 2, ctx->stream));
-            if (prof) {
-                CK(ctx, cudaEventRecord(ctx->gemm_ev[ctx->gemm_ev_used + 1], ctx->stream));
-                ctx->gemm_ev_used += 2;
-            }
+            CK(ctx, mark(1));
             ctx->gemm_launches += 1;
             ctx->gemm_flop += 2.0 * nf.n[k + 1] * nf.n[k] * ((double)nb * (2 * d + 1));
-            CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur], Kh, Kl, Ke, sms, ctx->stream));
+            CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur] + (size_t)(d + 1) * np, (int64_t)(d + 3) * np,
+                                           Kh, Kl, Ke, sms, ctx->stream));
             const float g = slr::tc_gamma(ctx->w_Kpad[k]);
             if (k + 1 < K) {
                 CK(ctx, slr::launch_wide_hidden(nf, k + 1, nb, np, g, Cb[nxt], Rb[nxt], Ch, Cl, Kh, Kl, Ke, src.alpha,
