@@ -124,7 +124,8 @@ struct slr_ctx {
     const float *wa_hi[slr::kMaxLayers] = {}, *wa_lo[slr::kMaxLayers] = {};
     const float *w0t = nullptr;           // layer 1 transposed (d x n_1)
     bool wide_layers = false;             // hidden layers by wide_layer_kernel
-    const float *w0p = nullptr;           // layer 1 transposed, rows padded with zeros (d x wide_NP)
+    int wide_cols = 0;                    // columns of a box's state: d, padded to its tiles there
+    const float *w0b = nullptr;           // layer 1 in the layer kernel's state layout of one box
     const unsigned char *w_img[slr::kMaxLayers] = {};   // its weight pieces per layer
     int w_Kpad[slr::kMaxLayers] = {};
     // transposed pieces (W_k^T, |W_k|^T) for the adjoint's backward products
@@ -574,8 +575,11 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
     // one kernel per hidden layer where its column tiles of one box are filled
     // by at least kWideLayerMinD inputs and the property's rows fit its product
     ctx->wide_layers = K > 1 && nf.R <= 16 && d >= slr::kWideLayerMinD;
-    const size_t off_w0p = total;
-    if (ctx->wide_layers) total += align_up((size_t)d * np * sizeof(float));
+    int ntile = 0, nc = 0;
+    if (ctx->wide_layers) slr::wide_layer_tiles(d, ntile, nc);
+    ctx->wide_cols = ctx->wide_layers ? ntile * nc : d;
+    const size_t off_w0b = total;
+    total += align_up((size_t)ntile * nc * np * sizeof(float));
     for (int k = 1; k < K; ++k) {
         const int Mpad = (nf.n[k + 1] + 127) & ~127, Kpad = (nf.n[k] + 31) & ~31;
         ctx->w_Kpad[k] = Kpad;
@@ -601,9 +605,11 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
         for (int p = 0; p < nf.n[1]; ++p)
             for (int j = 0; j < d; ++j) w0t[(size_t)j * nf.n[1] + p] = L.W[0][(size_t)p * d + j];
         if (ctx->wide_layers) {
-            float *w0p = (float *)(host.data() + off_w0p);
+            float *w0b = (float *)(host.data() + off_w0b);
             for (int j = 0; j < d; ++j)
-                std::memcpy(w0p + (size_t)j * np, w0t + (size_t)j * nf.n[1], nf.n[1] * sizeof(float));
+                for (int p0 = 0; p0 < nf.n[1]; p0 += 16)
+                    std::memcpy(w0b + ((size_t)(j / nc) * (np / 16) + p0 / 16) * nc * 16 + (size_t)(j % nc) * 16,
+                                w0t + (size_t)j * nf.n[1] + p0, std::min(16, nf.n[1] - p0) * sizeof(float));
         }
         for (int k = 1; k < K; ++k) {
             const int n_in = nf.n[k], n_out = nf.n[k + 1];
@@ -641,7 +647,7 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
         CK(ctx, cudaMemcpy(ctx->wide_img, host.data(), host_total, cudaMemcpyHostToDevice));
         ctx->h2d_pending += (int64_t)host_total;
         ctx->w0t = (const float *)ctx->wide_img;
-        ctx->w0p = (const float *)((const unsigned char *)ctx->wide_img + off_w0p);
+        ctx->w0b = (const float *)((const unsigned char *)ctx->wide_img + off_w0b);
         for (int k = 1; k < K; ++k) {
             const int Mpad = (nf.n[k + 1] + 127) & ~127;
             const size_t one = align_up((size_t)Mpad * ctx->w_Kpad[k] * sizeof(float));
@@ -677,13 +683,13 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
 
 int ensure_wide_buf(slr_ctx *ctx) {
     const int d = ctx->nf.d, np = ctx->wide_NP, R = ctx->nf.R;
-    const size_t bc = (size_t)ctx->wide_Bc;
-    size_t need = 2 * align_up(bc * d * np * 4) + 2 * align_up(bc * (d + 3) * np * 4) + 5 * align_up(bc * np * 4) +
+    const size_t bc = (size_t)ctx->wide_Bc, dc = (size_t)ctx->wide_cols;
+    size_t need = 2 * align_up(bc * dc * np * 4) + 2 * align_up(bc * (dc + 3) * np * 4) + 5 * align_up(bc * np * 4) +
                   3 * align_up(bc * d * 4) + 3 * align_up(bc * R * 4) + align_up(bc * 8);
     if (ctx->wide_layers) {
         int ntile, nc;
         slr::wide_layer_tiles(d, ntile, nc);
-        need += align_up(bc * 2 * np * 4) + 2 * align_up(bc * 3 * np * 4) + align_up(bc * 8 * ntile * np * 4);
+        need += align_up(bc * 2 * np * 4) + 2 * align_up(bc * 3 * np * 4) + align_up(bc * 12 * ntile * np * 4);
     }
     if (ctx->wide_buf_bytes >= need) return SLR_OK;
     cudaFree(ctx->wide_buf);
@@ -708,18 +714,21 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
         p += align_up(bytes);
         return q;
     };
-    float *Cb[2] = {take(bc * d * np * 4), take(bc * d * np * 4)};
-    float *Rb[2] = {take(bc * (d + 3) * np * 4), take(bc * (d + 3) * np * 4)};
+    const size_t dc = (size_t)ctx->wide_cols;
+    float *Cb[2] = {take(bc * dc * np * 4), take(bc * dc * np * 4)};
+    float *Rb[2] = {take(bc * (dc + 3) * np * 4), take(bc * (dc + 3) * np * 4)};
     float *Ch = take(bc * np * 4), *Cl = take(bc * np * 4);
     float *Kh = take(bc * np * 4), *Kl = take(bc * np * 4), *Ke = take(bc * np * 4);
     float *mh = take(bc * d * 4), *ml = take(bc * d * 4), *rr = take(bc * d * 4);
     float *lo = take(bc * R * 4), *hi = take(bc * R * 4), *er = take(bc * R * 4);
     int64_t *bidx = (int64_t *)take(bc * 8);
-    float *plan = nullptr, *S3 = nullptr, *T3 = nullptr, *part = nullptr;
+    // layer kernels: relaxations, the small columns of two layers, bound sums
+    float *plan = nullptr, *S3[2] = {}, *part = nullptr;
+    float *Hh[2] = {Ch, Kh}, *Hl[2] = {Cl, Kl};
     if (ctx->wide_layers) {
         plan = take(bc * 2 * np * 4);
-        S3 = take(bc * 3 * np * 4);
-        T3 = take(bc * 3 * np * 4);
+        S3[0] = take(bc * 3 * np * 4);
+        S3[1] = take(bc * 3 * np * 4);
         part = (float *)p;
     }
     const bool prof = ctx->opt.profile != 0;
@@ -736,13 +745,15 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
         if (after) ctx->gemm_ev_used += 2;
         return re;
     };
-    for (int64_t base = 0; base < n; base += (int64_t)bc) {
-        const int nb = (int)std::min<int64_t>((int64_t)bc, n - base);
+    // chunks of nearly equal size: a short last one would pay every kernel's latency for a few boxes
+    const int64_t chunks = (n + (int64_t)bc - 1) / (int64_t)bc, chunk = chunks > 0 ? (n + chunks - 1) / chunks : 1;
+    for (int64_t base = 0; base < n; base += chunk) {
+        const int nb = (int)std::min<int64_t>(chunk, n - base);
         CK(ctx, slr::launch_wide_box(src, base, nb, d, mh, ml, rr, bidx, sms, ctx->stream));
         int cur = 0;
         if (ctx->wide_layers) {
-            CK(ctx, slr::launch_wide_plan1(nf, ctx->w0p, nb, np, mh, ml, rr, plan, S3, Ch, Cl, src.alpha, src.alpha_ld,
-                                           base, ctx->stream));
+            CK(ctx, slr::launch_wide_plan1(nf, ctx->w0t, nb, np, mh, ml, rr, plan, S3[0], Hh[0], Hl[0], src.alpha,
+                                           src.alpha_ld, base, ctx->stream));
             *launches += 2;
             for (int k = 1; k + 1 < K; ++k) {
                 const int nxt = cur ^ 1;
@@ -750,7 +761,7 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
                 g.Aimg = ctx->w_img[k];
                 g.Cin = k > 1 ? Cb[cur] : nullptr;
                 g.Rin = k > 1 ? Rb[cur] : nullptr;
-                g.W0p = ctx->w0p;
+                g.W0b = ctx->w0b;
                 g.rr = rr;
                 g.plan = plan;
                 g.Cout = Cb[nxt];
@@ -764,35 +775,24 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
                 g.status = out.status;
                 CK(ctx, mark(0));
                 CK(ctx, slr::launch_wide_layer(g, sms, ctx->stream));
-                // the radius constant, N and E columns
-                slr::WideGemmArgs ga{};
-                ga.status = out.status;
-                ga.g[0] = slr::WideGemm{ctx->wa_hi[k], ctx->wa_lo[k], S3, T3, nf.n[k + 1], nf.n[k], ctx->w_Kpad[k],
-                                        3 * nb, np, np};
-                CK(ctx, slr::launch_wide_gemm(ga, 1, ctx->stream));
                 CK(ctx, mark(1));
                 ctx->gemm_launches += 1;
                 ctx->gemm_flop += 2.0 * nf.n[k + 1] * nf.n[k] * ((double)nb * (2 * d + 1));
-                CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, S3 + np, 3 * (int64_t)np, Kh, Kl, Ke, sms,
-                                               ctx->stream));
-                CK(ctx, slr::launch_wide_plan(nf, k + 1, nb, np, slr::tc_gamma(ctx->w_Kpad[k]), part, T3, Kh, Kl, Ke,
-                                              plan, S3, Ch, Cl, src.alpha, src.alpha_ld, base, ctx->stream));
-                *launches += 4;
+                CK(ctx, slr::launch_wide_plan(nf, k + 1, nb, np, slr::tc_gamma(ctx->w_Kpad[k]), part, S3[cur], Hh[cur],
+                                              Hl[cur], plan, S3[nxt], Hh[nxt], Hl[nxt], src.alpha, src.alpha_ld, base,
+                                              ctx->stream));
+                *launches += 2;
                 cur = nxt;
             }
             // the property layer: a few rows, on the CUDA cores
             const bool gen = K == 2;
             float *cols = Cb[cur ^ 1];
-            CK(ctx, slr::launch_wide_rows(nf, nb, np, gen ? nullptr : Cb[cur], gen ? nullptr : Rb[cur], ctx->w0p, rr,
+            CK(ctx, slr::launch_wide_rows(nf, nb, np, gen ? nullptr : Cb[cur], gen ? nullptr : Rb[cur], ctx->w0b, rr,
                                           plan, cols, sms, ctx->stream));
-            CK(ctx, slr::launch_wide_rows_product(nf.Wt[K - 1], nf.n[K - 1], R, S3, np, T3, np, 3 * (int64_t)nb, true,
-                                                  sms, ctx->stream));
-            CK(ctx, slr::launch_wide_const(nf, K - 1, nb, np, Ch, Cl, S3 + np, 3 * (int64_t)np, Kh, Kl, Ke, sms,
-                                           ctx->stream));
-            CK(ctx, slr::launch_wide_rows_final(nf, nb, np, (float)(nf.n[K - 1] + 2) * 0x1p-24f, cols, T3, Kh, Kl, Ke,
-                                                lo, hi, er, ctx->stream));
+            CK(ctx, slr::launch_wide_rows_final(nf, nb, np, (float)(nf.n[K - 1] + 2) * 0x1p-24f, cols, S3[cur], Hh[cur],
+                                                Hl[cur], lo, hi, er, ctx->stream));
             CK(ctx, slr::launch_wide_classify(nf, nb, base, lo, hi, er, bidx, out, sms, ctx->stream));
-            *launches += 5;
+            *launches += 3;
             continue;
         }
         CK(ctx, slr::launch_wide_init(nf, ctx->w0t, nb, np, mh, ml, rr, Cb[cur], Rb[cur], Ch, Cl, src.alpha,
@@ -807,8 +807,7 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
                                                       (int64_t)nb * d, false, sms, ctx->stream));
                 CK(ctx, slr::launch_wide_rows_product(nf.Wt[k], nf.n[k], nf.R, Rb[cur], np, Rb[nxt], np,
                                                       (int64_t)nb * (d + 3), true, sms, ctx->stream));
-                CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur] + (size_t)(d + 1) * np, (int64_t)(d + 3) * np,
-                                           Kh, Kl, Ke, sms, ctx->stream));
+                CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur], Kh, Kl, Ke, sms, ctx->stream));
                 const float gf = (float)(nf.n[k] + 2) * 0x1p-24f;
                 CK(ctx, slr::launch_wide_final(nf, nb, np, gf, Cb[nxt], Rb[nxt], Ch, Cl, Kh, Kl, Ke, lo, hi, er,
                                                ctx->stream));
@@ -827,8 +826,7 @@ int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::Eval
             CK(ctx, mark(1));
             ctx->gemm_launches += 1;
             ctx->gemm_flop += 2.0 * nf.n[k + 1] * nf.n[k] * ((double)nb * (2 * d + 1));
-            CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur] + (size_t)(d + 1) * np, (int64_t)(d + 3) * np,
-                                           Kh, Kl, Ke, sms, ctx->stream));
+            CK(ctx, slr::launch_wide_const(nf, k, nb, np, Ch, Cl, Rb[cur], Kh, Kl, Ke, sms, ctx->stream));
             const float g = slr::tc_gamma(ctx->w_Kpad[k]);
             if (k + 1 < K) {
                 CK(ctx, slr::launch_wide_hidden(nf, k + 1, nb, np, g, Cb[nxt], Rb[nxt], Ch, Cl, Kh, Kl, Ke, src.alpha,

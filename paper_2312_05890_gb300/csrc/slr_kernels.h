@@ -170,10 +170,8 @@ cudaError_t launch_wide_box(const BoxSource &src, int64_t base, int nb, int d, f
 cudaError_t launch_wide_init(const NetParams<float> &net, const float *W0t, int nb, int NP, const float *mh,
                              const float *ml, const float *rr, float *C, float *Rr, float *Ch, float *Cl,
                              const float *alpha, int64_t alpha_ld, int64_t base, cudaStream_t s);
-// NE: the rows' N at NE[b * ne_stride + p] and E at NE[b * ne_stride + NP + p].
 cudaError_t launch_wide_const(const NetParams<float> &net, int k, int nb, int NP, const float *Ch, const float *Cl,
-                              const float *NE, int64_t ne_stride, float *Kh, float *Kl, float *Ke, int sms,
-                              cudaStream_t s);
+                              const float *Rr, float *Kh, float *Kl, float *Ke, int sms, cudaStream_t s);
 cudaError_t launch_wide_hidden(const NetParams<float> &net, int layer, int nb, int NP, float gcoef, float *C, float *Rr,
                                float *Ch, float *Cl, const float *Kh, const float *Kl, const float *Ke,
                                const float *alpha, int64_t alpha_ld, int64_t base, cudaStream_t s);
@@ -187,13 +185,13 @@ cudaError_t launch_wide_classify(const NetParams<float> &net, int nb, int64_t ba
 // Wide networks of many inputs: one kernel per hidden layer (slr_wide_layer.cu).
 struct WideLayer {
     const unsigned char *Aimg;    // weight pieces as ring stages (launch_wide_pack)
-    const float *Cin, *Rin;       // raw state of the layer's input [b][j][NP]; Cin null: layer 1,
-    const float *W0p, *rr;        // whose rows are W0p[j][NP] (zero padded) times rr[b][j]
+    const float *Cin, *Rin;       // raw state of the layer's input [b][tile][NP / 16][NC][16]; Cin null:
+    const float *W0b, *rr;        // layer 1, whose rows are W0b (one box's layout, zero padded) times rr[b][j]
     const float *plan;            // [b][2][NP]: pp, qq of the input's rows (zeros past its width)
-    float *Cout, *Rout;           // raw state of the output [b][j][NP]
-    float *part;                  // [b][2 ntile][4][NP]: the output rows' bound sums SU, SL, NC, NR
+    float *Cout, *Rout;           // raw state of the output
+    float *part;                  // [b][3 ntile][4][NP]: the output rows' bound sums SU, SL, NC, NR
     int nb, d, NP, n_in, n_out;
-    int nst, mt, ntile, NC;       // set by launch_wide_layer: stages, row tiles, column tiles, columns
+    int nst, mt, ntile, NC, na;   // set by launch_wide_layer: stages, row tiles, column tiles, columns, weight ring
     unsigned int *status;
 };
 constexpr int kWideLayerMinD = 64;   // fewest inputs the layer kernel takes
@@ -203,19 +201,18 @@ int wide_rows_stride(int R);
 cudaError_t launch_wide_pack(const float *hi, const float *lo, const float *ahi, const float *alo, int ld, int n_in,
                              int n_out, void *out, cudaStream_t s);
 cudaError_t launch_wide_layer(WideLayer G, int sms, cudaStream_t s);
-cudaError_t launch_wide_plan1(const NetParams<float> &net, const float *W0p, int nb, int NP, const float *mh,
+cudaError_t launch_wide_plan1(const NetParams<float> &net, const float *W0t, int nb, int NP, const float *mh,
                               const float *ml, const float *rr, float *plan, float *S3, float *Ch, float *Cl,
                               const float *alpha, int64_t alpha_ld, int64_t base, cudaStream_t s);
 cudaError_t launch_wide_plan(const NetParams<float> &net, int layer, int nb, int NP, float gcoef, const float *part,
-                             const float *T3, const float *Kh, const float *Kl, const float *Ke, float *plan,
-                             float *S3, float *Ch, float *Cl, const float *alpha, int64_t alpha_ld, int64_t base,
-                             cudaStream_t s);
+                             const float *S3, const float *Ch, const float *Cl, float *plan, float *S3o, float *Cho,
+                             float *Clo, const float *alpha, int64_t alpha_ld, int64_t base, cudaStream_t s);
 cudaError_t launch_wide_rows(const NetParams<float> &net, int nb, int NP, const float *Cin, const float *Rin,
-                             const float *W0p, const float *rr, const float *plan, float *out, int sms,
+                             const float *W0b, const float *rr, const float *plan, float *out, int sms,
                              cudaStream_t s);
 cudaError_t launch_wide_rows_final(const NetParams<float> &net, int nb, int NP, float gcoef, const float *cols,
-                                   const float *T3, const float *Kh, const float *Kl, const float *Ke, float *lo,
-                                   float *hi, float *err, cudaStream_t s);
+                                   const float *S3, const float *Ch, const float *Cl, float *lo, float *hi, float *err,
+                                   cudaStream_t s);
 
 cudaError_t launch_init_count(uint64_t *codes0, LevelCounters *ctr, cudaStream_t s);
 cudaError_t launch_compact(const uint64_t *codes_in, const uint8_t *cls, uint64_t *codes_out,

@@ -226,8 +226,9 @@ wide_init_kernel(const NetParams<float> net, const float *W0t, int NP, const flo
 // property layer, the rounding of the folded weights).
 // ---------------------------------------------------------------------------
 __global__ void wide_const_kernel(const NetParams<float> net, int k, int nb, int NP, const float *Ch, const float *Cl,
-                                  const float *NE, int64_t ne_stride, float *Kh, float *Kl, float *Ke) {
+                                  const float *Rr, float *Kh, float *Kl, float *Ke) {
     using A = Arith<float>;
+    const int d = net.d;
     const int n_in = net.n[k];
     const int n_out = net.n[k + 1];
     const bool last = k + 1 == net.K;
@@ -248,8 +249,8 @@ __global__ void wide_const_kernel(const NetParams<float> net, int k, int nb, int
             e = A::fma_rn(w, l, e + (pe + se));
             a = a + fabsf(p1);
             if (last) {
-                const float nN = NE[b * ne_stride + i];
-                const float nE = NE[b * ne_stride + NP + i];
+                const float nN = Rr[((size_t)b * (d + 3) + d + 1) * NP + i];
+                const float nE = Rr[((size_t)b * (d + 3) + d + 2) * NP + i];
                 const float z = A::add_up(A::add_up(fabsf(nN), fabsf(h)), A::add_up(fabsf(l), fabsf(nE)));
                 f = A::add_up(f, A::mul_up(net.fold_err[p * n_in + i], z));
             }
@@ -751,10 +752,9 @@ cudaError_t launch_wide_init(const NetParams<float> &net, const float *W0t, int 
 }
 
 cudaError_t launch_wide_const(const NetParams<float> &net, int k, int nb, int NP, const float *Ch, const float *Cl,
-                              const float *NE, int64_t ne_stride, float *Kh, float *Kl, float *Ke, int sms,
-                              cudaStream_t s) {
-    wide_const_kernel<<<grid_for((int64_t)nb * net.n[k + 1], sms), 256, 0, s>>>(net, k, nb, NP, Ch, Cl, NE, ne_stride,
-                                                                                  Kh, Kl, Ke);
+                              const float *Rr, float *Kh, float *Kl, float *Ke, int sms, cudaStream_t s) {
+    wide_const_kernel<<<grid_for((int64_t)nb * net.n[k + 1], sms), 256, 0, s>>>(net, k, nb, NP, Ch, Cl, Rr, Kh, Kl,
+                                                                                  Ke);
     return cudaGetLastError();
 }
 
