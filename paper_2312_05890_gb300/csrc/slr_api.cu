@@ -63,6 +63,13 @@ struct BatchState {
     std::vector<cudaEvent_t> step_ev;    // recorded at the end of each level step (graph nodes)
 };
 
+namespace {
+struct TileChoice {
+    int T = 0, NT = 0, blocks = 0;
+    size_t smem = 0;
+};
+}  // namespace
+
 struct slr_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -89,6 +96,7 @@ struct slr_ctx {
     bool pairs_fit = false;   // the FP64 tile's footprint holds the float-float stage's planes
     size_t smem32 = 0, smem64 = 0;
     int grid32 = 0, grid64 = 0;
+    std::vector<TileChoice> small32;      // the FP32 tiles of 256 threads, ascending (few_tile)
     int grid64c = 0;   // > 0: the FP64 re-check on clusters (grid of that many CTAs)
     void *tc_buf = nullptr;               // tensor-core weight images
     slr::TcParams tcp{};
@@ -344,11 +352,6 @@ void layout_params(const Src *ctx, const HostLayers<Real> &L, unsigned char *dev
     p.relax_mode = ctx->opt.relax_mode;
     for (int k = 0; k + 1 < K; ++k) p.act[k] = (uint8_t)(k < (int)ctx->act.size() ? ctx->act[k] : slr::kActRelu);
 }
-
-struct TileChoice {
-    int T = 0, NT = 0, blocks = 0;
-    size_t smem = 0;
-};
 
 // Every (boxes per CTA, threads per CTA) the fused kernel can run this network with.
 // pairs (float64): with the planes of the float-float re-check stage.
@@ -967,32 +970,17 @@ int run_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int grid, int64_t *launches
 }
 
 // FP64 re-check of a list of boxes at level t: on clusters where chosen (pass
-// 1); else, with recheck_pairs, the float-float stage (pass 2) lists the
-// boxes it leaves depending on E in the other re-check list, and pass 1
-// re-bounds those with plain FP64 products.  Returns the launches in *n.
-cudaError_t launch_recheck(slr_ctx *ctx, const slr::BoxSource &src, const slr::EvalOutputs &out, int t,
-                           int64_t *n) {
-    *n = 1;
+// 1); else, with recheck_pairs, the float-float stage (pass 2), after which a
+// tile that still holds boxes depending on E is bounded again with plain FP64
+// products by the same CTA; else plain FP64 products (pass 1).
+cudaError_t launch_recheck(slr_ctx *ctx, const slr::BoxSource &src, const slr::EvalOutputs &out, int t) {
     if (ctx->grid64c > 0)
         return slr::launch_eval_f64_cluster(ctx->T64, ctx->grid64c, ctx->smem64, ctx->stream, ctx->nd, src, out, 1);
-    if (ctx->opt.recheck_pairs && ctx->pairs_fit) {
-        int64_t *rest = src.index == ctx->near_list ? ctx->near_list2 : ctx->near_list;
-        slr::EvalOutputs oa = out;
-        oa.near_list = rest;
-        oa.near_count = &ctx->ctr->near3_n[t];
-        oa.near_cap = ctx->near_cap;
-        oa.tie_count = nullptr;
-        cudaError_t e =
-            slr::launch_eval_f64(ctx->T64, ctx->NT64, ctx->grid64, ctx->smem64, ctx->stream, ctx->nd, src, oa, 2);
-        if (e != cudaSuccess) return e;
-        slr::BoxSource sb = src;
-        sb.index = rest;
-        sb.index_count = &ctx->ctr->near3_n[t];
-        sb.cap = ctx->near_cap;
-        *n = 2;
-        return slr::launch_eval_f64(ctx->T64, ctx->NT64, ctx->grid64, ctx->smem64, ctx->stream, ctx->nd, sb, out, 1);
-    }
-    return slr::launch_eval_f64(ctx->T64, ctx->NT64, ctx->grid64, ctx->smem64, ctx->stream, ctx->nd, src, out, 1);
+    slr::EvalOutputs o = out;
+    const bool pairs = ctx->opt.recheck_pairs && ctx->pairs_fit;
+    if (pairs) o.near_count = &ctx->ctr->near3_n[t];
+    return slr::launch_eval_f64(ctx->T64, ctx->NT64, ctx->grid64, ctx->smem64, ctx->stream, ctx->nd, src, o,
+                                pairs ? 2 : 1);
 }
 
 // FP64 re-check: short lists, so the smallest tiles spread them over the
@@ -1014,6 +1002,22 @@ std::vector<TileChoice> recheck_candidates(slr_ctx *ctx, bool pairs) {
     }
     return c64;
 }
+
+// The FP32 tile for at most `most` boxes: the smallest tile that still gives
+// every tile an SM of its own, else the context's.  A tile's time grows with
+// its boxes, so few boxes are done soonest on many small tiles: levels 0 to 8
+// of a 5-6x50-5 tanh count take 45 us each on 4-box tiles, 78 us on its 20-box
+// one, the whole depth-16 count 3.66 -> 3.22 ms.  The rule
+// takes nothing but the boxes and the context's tile: a level of a count (at
+// most 2^t boxes) runs the same tile in every form of the count.
+TileChoice few_tile(const slr_ctx *ctx, int64_t most) {
+    for (const TileChoice &c : ctx->small32) {
+        if (c.T >= ctx->T32) break;
+        if ((most + c.T - 1) / c.T <= ctx->sm_count) return c;
+    }
+    return TileChoice{ctx->T32, ctx->NT32, ctx->grid32 / std::max(1, ctx->sm_count), ctx->smem32};
+}
+TileChoice level_tile(const slr_ctx *ctx, int t) { return few_tile(ctx, (int64_t)1 << std::min(t, 40)); }
 
 void choose_recheck_tile(slr_ctx *ctx) {
     std::vector<TileChoice> c64 = recheck_candidates(ctx, true);
@@ -1118,6 +1122,9 @@ int prepare_device(slr_ctx *ctx) {
     ctx->NT32 = best.NT;
     ctx->smem32 = best.smem;
     ctx->grid32 = best.blocks * ctx->sm_count;
+    ctx->small32.clear();
+    for (auto c = c32.rbegin(); c != c32.rend(); ++c)
+        if (c->NT == 256) ctx->small32.push_back(*c);
     choose_recheck_tile(ctx);
     // adjoint: keep as many hidden layers' equations in shared memory as fit in
     // 96 KB, recompute the others
@@ -1273,12 +1280,10 @@ int slr_internal_noalloc_view(slr_ctx *ctx, slr_noalloc_view *v) {
     v->d = ctx->widths[0];
     v->T32 = ctx->T32;
     v->NT32 = ctx->NT32;
-    v->grid32 = ctx->grid32;
     v->T64 = ctx->T64;
     v->NT64 = ctx->NT64;
     v->grid64 = ctx->grid64;
     v->sm_count = ctx->sm_count;
-    v->smem32 = ctx->smem32;
     v->smem64 = ctx->smem64;
     v->nf = &ctx->nf;
     v->nd = &ctx->nd;
@@ -1288,6 +1293,14 @@ int slr_internal_noalloc_view(slr_ctx *ctx, slr_noalloc_view *v) {
     v->ev0 = ctx->ev0;
     v->ev1 = ctx->ev1;
     return SLR_OK;
+}
+
+void slr_internal_level_tile(const slr_ctx *ctx, int t, int *T, int *NT, int *grid, size_t *smem) {
+    const TileChoice c = level_tile(ctx, t);
+    *T = c.T;
+    *NT = c.NT;
+    *grid = c.blocks * ctx->sm_count;
+    *smem = c.smem;
 }
 
 int slr_internal_fail(slr_ctx *ctx, int code, const char *msg) { return fail(ctx, code, "%s", msg); }
@@ -1702,9 +1715,8 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
                 o2.cls = ctx->cls;
                 o2.tie_count = &ctx->ctr->ties;
                 o2.status = ctx->status;
-                int64_t nl = 0;
-                CK(ctx, launch_recheck(ctx, s2, o2, t, &nl));
-                launches += nl;
+                CK(ctx, launch_recheck(ctx, s2, o2, t));
+                ++launches;
             }
         } else if (use_tc) {
             // tier 1 on the tensor cores; boxes whose class depends on its
@@ -1732,12 +1744,13 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
                 o2.cls = ctx->cls;
                 o2.tie_count = &ctx->ctr->ties;
                 o2.status = ctx->status;
-                int64_t nl = 0;
-                CK(ctx, launch_recheck(ctx, s2, o2, t, &nl));
-                launches += nl;
+                CK(ctx, launch_recheck(ctx, s2, o2, t));
+                ++launches;
             }
         } else {
-        CK(ctx, slr::launch_eval_f32(ctx->T32, ctx->NT32, ctx->grid32, ctx->smem32, ctx->stream, ctx->nf, src, o, 0));
+        const TileChoice tile = level_tile(ctx, t);
+        CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, tile.blocks * ctx->sm_count, tile.smem, ctx->stream, ctx->nf, src,
+                                     o, 0));
         CK(ctx, mark(t, 1));
         ++launches;
         if (recheck) {
@@ -1749,9 +1762,8 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
             o2.cls = ctx->cls;
             o2.tie_count = &ctx->ctr->ties;
             o2.status = ctx->status;
-            int64_t nl = 0;
-            CK(ctx, launch_recheck(ctx, s2, o2, t, &nl));
-            launches += nl;
+            CK(ctx, launch_recheck(ctx, s2, o2, t));
+            ++launches;
         }
         }
         CK(ctx, mark(t, 2));
@@ -1770,7 +1782,7 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
                                     ctx->leaf_cls, ctx->opt.leaf_cap, compact_grid, ctx->stream, path_mask,
                                     !sharded || ctx->opt.shard_index == 0 || t >= shard_g));
         CK(ctx, mark(t, 5));
-        launches += 2;
+        launches += slr::compact_launches(t);
     }
     return SLR_OK;
     };
@@ -2300,9 +2312,9 @@ int slr_bounds(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi
         const int grid = (int)std::min<int64_t>(tiles, ctx->grid_tc);
         CK(ctx, slr::launch_eval_tc(ctx->T_tc, grid, ctx->smem_tc, ctx->stream, ctx->nf, ctx->tcp, src, o, 0));
     } else {
-        const int64_t tiles = (n + ctx->T32 - 1) / ctx->T32;
-        const int grid = (int)std::min<int64_t>(tiles, ctx->grid32);
-        CK(ctx, slr::launch_eval_f32(ctx->T32, ctx->NT32, grid, ctx->smem32, ctx->stream, ctx->nf, src, o, 0));
+        const TileChoice tile = few_tile(ctx, n);
+        const int grid = (int)std::min<int64_t>((n + tile.T - 1) / tile.T, (int64_t)tile.blocks * ctx->sm_count);
+        CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, grid, tile.smem, ctx->stream, ctx->nf, src, o, 0));
     }
     if (!on_device) {
         if (row_lo) {
@@ -3135,9 +3147,10 @@ int eval_by_position(slr_ctx *ctx, slr::BoxSource src, const float *alpha, float
         int64_t launches = 0;
         return n > 0 ? run_wide(ctx, src, n, o, &launches) : SLR_OK;
     }
-    const int64_t tiles = (n_hint + ctx->T32 - 1) / ctx->T32;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, ctx->grid32));
-    CK(ctx, slr::launch_eval_f32(ctx->T32, ctx->NT32, grid, ctx->smem32, ctx->stream, ctx->nf, src, o, 0));
+    const TileChoice tile = few_tile(ctx, n_hint);
+    const int64_t tiles = (n_hint + tile.T - 1) / tile.T;
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)tile.blocks * ctx->sm_count));
+    CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, grid, tile.smem, ctx->stream, ctx->nf, src, o, 0));
     return SLR_OK;
 }
 

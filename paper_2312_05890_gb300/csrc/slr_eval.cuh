@@ -1603,14 +1603,17 @@ __device__ __forceinline__ int64_t source_count(const BoxSource &src) {
 // pass 0: working precision; writes the sound class and lists the undecided
 //         boxes whose class depends on E (their optimistic class differs);
 // pass 2: float64 with float-float hidden products (see contract_ff): writes
-//         the class and lists the boxes whose class still depends on E;
+//         the class, counts the boxes whose class still depends on E and
+//         marks them in near_mask (64 bits: place in the tile);
 // pass 1: re-check of such a list in the higher precision (writes the class,
-//         counts the boxes still depending on E as ties).
+//         counts the boxes still depending on E as ties); `only` non-zero:
+//         of these boxes of the tile.
 // ---------------------------------------------------------------------------
 // kPairs: pass 2 is compiled in (the single-problem float64 kernel).
 template <typename Real, int T, int NT, int KI = 2, int CL = 1, int DC = 0, bool kPairs = false>
 __device__ void eval_tile(const NetParams<Real> &net, const BoxSource &src, const EvalOutputs &out, const int pass,
-                          const TileSmem<Real> &sm, const int64_t base, const int64_t n) {
+                          const TileSmem<Real> &sm, const int64_t base, const int64_t n,
+                          unsigned *near_mask = nullptr, const unsigned long long only = 0ull) {
     using A = Arith<Real>;
     using Tile = EvalTile<Real, T, NT, KI, DC>;
     const int d = Tile::dim_of(net);
@@ -1744,7 +1747,8 @@ __device__ void eval_tile(const NetParams<Real> &net, const BoxSource &src, cons
     __syncthreads();
 
     // ---- classify (Sec. 3) and write (one CTA of a cluster) ----------------
-    if (threadIdx.x < nb && (CL == 1 || cluster_ctarank() == 0)) {
+    if (threadIdx.x < nb && (CL == 1 || cluster_ctarank() == 0) &&
+        (only == 0ull || (only >> threadIdx.x & 1ull) != 0ull)) {
         const int b = threadIdx.x;
         const uint8_t cls = classify_rows<Real, T>(net, sLo, sHi, sErr, b, (Real)0);
         // optimistic bounds (raw +- E inward): the class the exact SLR could have
@@ -1763,7 +1767,10 @@ __device__ void eval_tile(const NetParams<Real> &net, const BoxSource &src, cons
             for (int r = 0; r < R; ++r) out.row_err[oidx * R + r] = to_hi<Real>(sErr[r * T + b]);
         }
         if (near) {
-            if ((pass == 0 || pass == 2) && out.near_list != nullptr) {
+            if (kPairs && pass == 2) {
+                atomicAdd(out.near_count, 1ull);
+                atomicOr(near_mask + (b >> 5), 1u << (b & 31));
+            } else if (pass == 0 && out.near_list != nullptr) {
                 const unsigned long long pos = atomicAdd(out.near_count, 1ull);
                 if ((int64_t)pos < out.near_cap) {
                     out.near_list[pos] = idx;
@@ -1796,8 +1803,22 @@ slr_eval_kernel(const NetParams<Real> net, const BoxSource src, const EvalOutput
     const TileSmem<Real> sm =
         carve_smem<Real, T>(smem_raw, net.n_max_pad, DC > 0 ? DC : net.d, net.n_in_max, net.R);
     const int64_t n = source_count(src);
-    for (int64_t base = (int64_t)blockIdx.x * T; base < n; base += (int64_t)gridDim.x * T)
-        eval_tile<Real, T, NT, KI, 1, DC, sizeof(Real) == 8>(net, src, out, pass, sm, base, n);
+    for (int64_t base = (int64_t)blockIdx.x * T; base < n; base += (int64_t)gridDim.x * T) {
+        if constexpr (sizeof(Real) == 8) {
+            // what the float-float stage leaves depending on E goes on to plain products
+            unsigned *near = reinterpret_cast<unsigned *>(sm.sNRows) + 1;   // (two words, in the footprint's slack)
+            if (threadIdx.x < 2) near[threadIdx.x] = 0u;   // (the tile's first barrier precedes its marks)
+            unsigned long long only = 0ull;
+            for (int ps = pass;; ps = 1) {
+                eval_tile<Real, T, NT, KI, 1, DC, true>(net, src, out, ps, sm, base, n, near, only);
+                only = near[0] | (unsigned long long)near[1] << 32;   // (the tile ends with a barrier)
+                if (ps != 2 || only == 0ull) break;
+            }
+            __syncthreads();
+        } else {
+            eval_tile<Real, T, NT, KI, 1, DC>(net, src, out, pass, sm, base, n);
+        }
+    }
 }
 
 // The float64 re-check with each tile on a cluster of kRecheckCluster CTAs (one

@@ -215,6 +215,9 @@ cudaError_t launch_wide_rows_final(const NetParams<float> &net, int nb, int NP, 
                                    cudaStream_t s);
 
 cudaError_t launch_init_count(uint64_t *codes0, LevelCounters *ctr, cudaStream_t s);
+// Kernels launch_compact runs at level t (at most 2^t boxes): one block where
+// the level holds at most 4096 boxes, else a counting and a writing pass.
+inline int compact_launches(int t) { return t <= 12 ? 1 : 2; }
 cudaError_t launch_compact(const uint64_t *codes_in, const uint8_t *cls, uint64_t *codes_out,
                            LevelCounters *ctr, unsigned int *status, int64_t cap, int t, int D,
                            uint64_t *leaf_codes, uint8_t *leaf_depth, uint8_t *leaf_cls,

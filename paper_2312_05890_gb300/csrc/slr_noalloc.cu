@@ -139,7 +139,10 @@ extern "C" int slr_count_noalloc(slr_ctx *ctx, int D, slr_result *out) {
         o.near_cap = kNearCap;
         o.tie_count = &ctr->ties;
         o.status = status;
-        NA_CK(slr::launch_eval_f32(v.T32, v.NT32, v.grid32, v.smem32, s, *v.nf, src, o, 0));
+        int T, NT, grid;
+        size_t smem;
+        slr_internal_level_tile(ctx, t, &T, &NT, &grid, &smem);
+        NA_CK(slr::launch_eval_f32(T, NT, grid, smem, s, *v.nf, src, o, 0));
         ++launches;
         if (recheck) {
             slr::BoxSource s2 = src;
@@ -155,7 +158,7 @@ extern "C" int slr_count_noalloc(slr_ctx *ctx, int D, slr_result *out) {
         }
         NA_CK(slr::launch_compact(codes[t & 1], cls, codes[(t + 1) & 1], ctr, status, kFrontierCap, t, D, nullptr,
                                   nullptr, nullptr, 0, v.sm_count * 4, s));
-        launches += 2;
+        launches += slr::compact_launches(t);
     }
     NA_CK(cudaEventRecord(v.ev1, s));
     slr::LevelCounters c;

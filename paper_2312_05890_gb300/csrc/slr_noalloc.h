@@ -10,8 +10,8 @@ struct slr_noalloc_view {
     int device;
     cudaStream_t stream;
     int d;
-    int T32, NT32, grid32, T64, NT64, grid64, sm_count;
-    size_t smem32, smem64;
+    int T32, NT32, T64, NT64, grid64, sm_count;
+    size_t smem64;
     const slr::NetParams<float> *nf;
     const slr::NetParams<double> *nd;
     const float *lo, *hi;
@@ -22,5 +22,7 @@ struct slr_noalloc_view {
 // Fills *v when the network and property are resident on the device
 // (SLR_ESTATE otherwise); allocates nothing.
 int slr_internal_noalloc_view(slr_ctx *ctx, slr_noalloc_view *v);
+// The FP32 tile slr_count runs level t on.
+void slr_internal_level_tile(const slr_ctx *ctx, int t, int *T, int *NT, int *grid, size_t *smem);
 // Records `msg` as the context's last error and returns `code`.
 int slr_internal_fail(slr_ctx *ctx, int code, const char *msg);
