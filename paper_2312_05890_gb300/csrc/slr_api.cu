@@ -88,8 +88,10 @@ struct slr_ctx {
     std::vector<int> act;                 // activation after each hidden layer (empty: ReLU)
     bool has_net = false, has_box = false, has_prop = false;
 
-    bool dev_dirty = true;
+    bool dev_dirty = true;                // network or property not on the device as set
+    bool net_dirty = true;                // more than the property changed since prepare_device
     void *net_buf = nullptr;
+    size_t prop32 = 0, prop64 = 0, net_bytes = 0;   // in net_buf: the property's arrays, its size
     slr::NetParams<float> nf{};
     slr::NetParams<double> nd{};
     int T32 = 0, T64 = 0, NT32 = 0, NT64 = 0;
@@ -214,8 +216,9 @@ bool finite_all(const float *p, size_t n) {
 // Fold the property rows into the last layer in float64 (Sec. 3 check on the
 // rows C y + e): W' = C W_K, b' = C b_K + e, with a bound on the float64
 // rounding error, then round to the working precision and add that rounding.
+// prop_only: the last layer alone (what a new property changes).
 template <typename Real, typename Src>
-void build_layers(const Src *ctx, HostLayers<Real> &L) {
+void build_layers(const Src *ctx, HostLayers<Real> &L, bool prop_only = false) {
     const int K = ctx->K;
     const int R = (int)ctx->e.size();
     const int n_out = ctx->widths[K];
@@ -247,7 +250,7 @@ void build_layers(const Src *ctx, HostLayers<Real> &L) {
     }
     L.W.assign(K, {});
     L.b.assign(K, {});
-    for (int k = 0; k < K; ++k) {
+    for (int k = prop_only ? K - 1 : 0; k < K; ++k) {
         const int ni = ctx->widths[k];
         const bool last = k == K - 1;
         const int no = last ? R : ctx->widths[k + 1];
@@ -276,7 +279,7 @@ void build_layers(const Src *ctx, HostLayers<Real> &L) {
         L.fold_berr[r] = sizeof(Real) == 4 ? (Real)round_up_to_float(tot * (1 + 1e-15)) : (Real)(tot * (1 + 1e-15));
     }
     L.Ws.assign(K, {});
-    for (int k = 1; k < K; ++k) {
+    for (int k = prop_only ? std::max(1, K - 1) : 1; k < K; ++k) {
         const int ni = ctx->widths[k];
         const int no = k == K - 1 ? R : ctx->widths[k + 1];
         const int mp = (no + 7) & ~7;
@@ -303,9 +306,44 @@ size_t layers_bytes(const HostLayers<Real> &L) {
     return s;
 }
 
+// What a property decides of the parameters: the folded last layer, its bounds
+// and the clauses.  Arrays go to host + off (and dev + off on the device).
+template <typename Real, typename Src>
+void layout_property(const Src *ctx, const HostLayers<Real> &L, unsigned char *dev, unsigned char *host, size_t &off,
+                     slr::NetParams<Real> &p) {
+    auto put = [&](const std::vector<Real> &v) -> const Real * {
+        const Real *dp = reinterpret_cast<const Real *>(dev + off);
+        std::memcpy(host + off, v.data(), v.size() * sizeof(Real));
+        off += align_up(v.size() * sizeof(Real));
+        return dp;
+    };
+    const int K = ctx->K;
+    if (K == 1) {
+        p.W0 = put(L.W[0]);
+    } else {
+        p.Wt[K - 1] = put(L.W[K - 1]);
+        p.Ws[K - 1] = put(L.Ws[K - 1]);
+    }
+    p.fold_pad = L.fold_pad ? 1 : 0;
+    p.b[K - 1] = put(L.b[K - 1]);
+    p.fold_err = put(L.fold_err);
+    p.fold_berr = put(L.fold_berr);
+    p.n_clauses = ctx->n_clauses;
+    std::memset(p.clause_end, 0, sizeof p.clause_end);
+    std::memset(p.strict, 0, sizeof p.strict);
+    int end = 0;
+    for (int c = 0; c < ctx->n_clauses; ++c) {
+        end += ctx->rpc[c];
+        p.clause_end[c] = end;
+    }
+    for (int r = 0; r < p.R; ++r) p.strict[r] = ctx->strict[r];
+}
+
+// All parameters: what the network decides, then, from *prop_off on, what the
+// property does.
 template <typename Real, typename Src>
 void layout_params(const Src *ctx, const HostLayers<Real> &L, unsigned char *dev, unsigned char *host,
-                   size_t &off, slr::NetParams<Real> &p) {
+                   size_t &off, slr::NetParams<Real> &p, size_t *prop_off = nullptr) {
     auto put = [&](const std::vector<Real> &v) -> const Real * {
         const Real *dp = reinterpret_cast<const Real *>(dev + off);
         std::memcpy(host + off, v.data(), v.size() * sizeof(Real));
@@ -324,33 +362,22 @@ void layout_params(const Src *ctx, const HostLayers<Real> &L, unsigned char *dev
     for (int k = 1; k < K; ++k) nin = std::max(nin, p.n[k]);
     p.n_max_pad = (nmax + 7) & ~7;
     p.n_in_max = std::max(nin, 1);
-    p.W0 = put(L.W[0]);
-    for (int k = 1; k < K; ++k) p.Wt[k] = put(L.W[k]);
-    for (int k = 1; k < K; ++k) p.Ws[k] = put(L.Ws[k]);
-    p.fold_pad = L.fold_pad ? 1 : 0;
+    if (K > 1) p.W0 = put(L.W[0]);
+    for (int k = 1; k + 1 < K; ++k) p.Wt[k] = put(L.W[k]);
+    for (int k = 1; k + 1 < K; ++k) p.Ws[k] = put(L.Ws[k]);
     // hidden -> hidden: max_p sum_i |W[p][i]| (float64 sums of float weights, widened)
     for (int k = 1; k + 1 < K; ++k) {
         const int ni = p.n[k], no = p.n[k + 1];
-        double m = 0.0;
-        for (int q = 0; q < no; ++q) {
-            double a = 0.0;
-            for (int i = 0; i < ni; ++i) a += std::fabs((double)L.W[k][(size_t)i * no + q]);
-            m = std::max(m, a);
-        }
-        p.wabs[k] = m * (1.0 + 1e-12) + 1e-300;
+        std::vector<double> a(no, 0.0);
+        for (int i = 0; i < ni; ++i)
+            for (int q = 0; q < no; ++q) a[q] += std::fabs((double)L.W[k][(size_t)i * no + q]);
+        p.wabs[k] = *std::max_element(a.begin(), a.end()) * (1.0 + 1e-12) + 1e-300;
     }
-    for (int k = 0; k < K; ++k) p.b[k] = put(L.b[k]);
-    p.fold_err = put(L.fold_err);
-    p.fold_berr = put(L.fold_berr);
-    p.n_clauses = ctx->n_clauses;
-    int end = 0;
-    for (int c = 0; c < ctx->n_clauses; ++c) {
-        end += ctx->rpc[c];
-        p.clause_end[c] = end;
-    }
-    for (int r = 0; r < p.R; ++r) p.strict[r] = ctx->strict[r];
+    for (int k = 0; k + 1 < K; ++k) p.b[k] = put(L.b[k]);
     p.relax_mode = ctx->opt.relax_mode;
     for (int k = 0; k + 1 < K; ++k) p.act[k] = (uint8_t)(k < (int)ctx->act.size() ? ctx->act[k] : slr::kActRelu);
+    if (prop_off) *prop_off = off;
+    layout_property(ctx, L, dev, host, off, p);
 }
 
 // Every (boxes per CTA, threads per CTA) the fused kernel can run this network with.
@@ -563,6 +590,32 @@ int autotune(slr_ctx *ctx, const std::vector<TileChoice> &cands, TileChoice &bes
     return SLR_OK;
 }
 
+// The TF32 pieces [hi | lo | |hi| | signed lo] of layer k's weights at fwd (rows
+// of Kpad floats) and of their transpose at bwd (rows of KpadT), zeroed before.
+void fill_pieces(const HostLayers<float> &L, int k, int n_in, int n_out, int Kpad, int KpadT, unsigned char *fwd,
+                 unsigned char *bwd) {
+    const size_t one = align_up((size_t)((n_out + 127) & ~127) * Kpad * sizeof(float));
+    const size_t oneT = align_up((size_t)((n_in + 127) & ~127) * KpadT * sizeof(float));
+    float *f[4], *t[4];
+    for (int q = 0; q < 4; ++q) {
+        f[q] = (float *)(fwd + q * one);
+        t[q] = (float *)(bwd + q * oneT);
+    }
+    for (int p = 0; p < n_out; ++p) {
+        for (int i = 0; i < n_in; ++i) {
+            const float v = L.W[k][(size_t)i * n_out + p];   // transposed float weights
+            const float h = tf32_host(v);
+            const float l = tf32_host(v - h);
+            const float piece[4] = {h, l, std::fabs(h), v >= 0.f ? l : -l};
+            const size_t o = (size_t)p * Kpad + i, ot = (size_t)i * KpadT + p;
+            for (int q = 0; q < 4; ++q) {
+                f[q][o] = piece[q];
+                t[q][ot] = piece[q];
+            }
+        }
+    }
+}
+
 // Wide path: TF32 pieces of W and |W| of every layer k >= 1 (the last one
 // folded with the property), zero padded to multiples of 128 rows and 32
 // columns, and the chunk size for the per-box state.
@@ -617,34 +670,8 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
         for (int k = 1; k < K; ++k) {
             const int n_in = nf.n[k], n_out = nf.n[k + 1];
             const int Mpad = (n_out + 127) & ~127, Kpad = ctx->w_Kpad[k];
-            const size_t one = align_up((size_t)Mpad * Kpad * sizeof(float));
-            float *hi = (float *)(host.data() + offs[k]);
-            float *lo = (float *)(host.data() + offs[k] + one);
-            float *ahi = (float *)(host.data() + offs[k] + 2 * one);
-            float *alo = (float *)(host.data() + offs[k] + 3 * one);
-            const int KpadT = ctx->wt_Kpad[k];
-            const size_t oneT = align_up((size_t)((n_in + 127) & ~127) * KpadT * sizeof(float));
-            float *thi = (float *)(host.data() + offs_t[k]);
-            float *tlo = (float *)(host.data() + offs_t[k] + oneT);
-            float *tahi = (float *)(host.data() + offs_t[k] + 2 * oneT);
-            float *talo = (float *)(host.data() + offs_t[k] + 3 * oneT);
-            for (int p = 0; p < n_out; ++p) {
-                for (int i = 0; i < n_in; ++i) {
-                    const float v = L.W[k][(size_t)i * n_out + p];   // transposed float weights
-                    const float h = tf32_host(v);
-                    const float l = tf32_host(v - h);
-                    const size_t o = (size_t)p * Kpad + i;
-                    hi[o] = h;
-                    lo[o] = l;
-                    ahi[o] = std::fabs(h);
-                    alo[o] = v >= 0.f ? l : -l;
-                    const size_t ot = (size_t)i * KpadT + p;
-                    thi[ot] = h;
-                    tlo[ot] = l;
-                    tahi[ot] = std::fabs(h);
-                    talo[ot] = v >= 0.f ? l : -l;
-                }
-            }
+            (void)Mpad;
+            fill_pieces(L, k, n_in, n_out, Kpad, ctx->wt_Kpad[k], host.data() + offs[k], host.data() + offs_t[k]);
         }
         CK(ctx, cudaMalloc(&ctx->wide_img, total));
         CK(ctx, cudaMemcpy(ctx->wide_img, host.data(), host_total, cudaMemcpyHostToDevice));
@@ -1042,12 +1069,60 @@ void choose_recheck_tile(slr_ctx *ctx) {
     }
 }
 
+// A new property of as many rows for the network on the device: its arrays
+// alone are built and uploaded; tiles, tuning and buffers stay.  (A session
+// that checks many properties of one network pays this for each: the whole
+// network's layers took 2.8 ms of a 784-3x256-10 query, 64 us of a 2-8-8-1 one.)
+int new_property(slr_ctx *ctx) {
+    const int K = ctx->K;
+    HostLayers<float> Lf;
+    HostLayers<double> Ld;
+    build_layers(ctx, Lf, true);
+    build_layers(ctx, Ld, true);
+    const size_t c_bytes = align_up(ctx->C.size() * sizeof(float));
+    // the wide path's pieces of the last layer
+    const int n_in = ctx->nf.n[K - 1], n_out = ctx->nf.n[K];
+    size_t fwd = 0, bwd = 0;
+    if (ctx->wide) {
+        fwd = 4 * align_up((size_t)((n_out + 127) & ~127) * ctx->w_Kpad[K - 1] * sizeof(float));
+        bwd = 4 * align_up((size_t)((n_in + 127) & ~127) * ctx->wt_Kpad[K - 1] * sizeof(float));
+    }
+    CK(ctx, cudaStreamSynchronize(ctx->stream));   // the staging buffer and the arrays are not in use
+    int rc = ensure_stage(ctx, ctx->net_bytes + fwd + bwd);
+    if (rc) return rc;
+    unsigned char *dev = (unsigned char *)ctx->net_buf, *host = ctx->h_stage;
+    size_t off = ctx->prop32;
+    layout_property(ctx, Lf, dev, host, off, ctx->nf);
+    const size_t end32 = off;
+    off = ctx->prop64;
+    layout_property(ctx, Ld, dev, host, off, ctx->nd);
+    std::memcpy(host + off, ctx->C.data(), ctx->C.size() * sizeof(float));
+    off += c_bytes;
+    CK(ctx, cudaMemcpyAsync(dev + ctx->prop32, host + ctx->prop32, end32 - ctx->prop32, cudaMemcpyHostToDevice,
+                            ctx->stream));
+    CK(ctx, cudaMemcpyAsync(dev + ctx->prop64, host + ctx->prop64, off - ctx->prop64, cudaMemcpyHostToDevice,
+                            ctx->stream));
+    ctx->h2d_pending += (int64_t)(end32 - ctx->prop32 + off - ctx->prop64 + fwd + bwd);
+    if (ctx->wide) {
+        unsigned char *pf = host + ctx->net_bytes, *pb = pf + fwd;
+        std::memset(pf, 0, fwd + bwd);
+        fill_pieces(Lf, K - 1, n_in, n_out, ctx->w_Kpad[K - 1], ctx->wt_Kpad[K - 1], pf, pb);
+        CK(ctx, cudaMemcpyAsync((void *)ctx->w_hi[K - 1], pf, fwd, cudaMemcpyHostToDevice, ctx->stream));
+        CK(ctx, cudaMemcpyAsync((void *)ctx->wt_hi[K - 1], pb, bwd, cudaMemcpyHostToDevice, ctx->stream));
+    }
+    CK(ctx, cudaStreamSynchronize(ctx->stream));
+    ctx->dev_dirty = false;
+    return SLR_OK;
+}
+
 int prepare_device(slr_ctx *ctx) {
     if (!ctx->dev_dirty) return SLR_OK;
-    ctx->adjw_stale = true;
     if (ctx->widths.back() != (int)(ctx->C.size() / std::max<size_t>(1, ctx->e.size())))
         return fail(ctx, SLR_EINVAL, "property has %zu outputs per row but the network has %d outputs",
                     ctx->C.size() / std::max<size_t>(1, ctx->e.size()), ctx->widths.back());
+    if (!ctx->net_dirty && ctx->net_buf && ctx->K > 1 && ctx->nf.R == (int)ctx->e.size()) return new_property(ctx);
+    ctx->net_dirty = true;
+    ctx->adjw_stale = true;
     HostLayers<float> Lf;
     HostLayers<double> Ld;
     build_layers(ctx, Lf);
@@ -1064,8 +1139,9 @@ int prepare_device(slr_ctx *ctx) {
     if (rc) return rc;
     std::memset(ctx->h_stage, 0, bytes);
     size_t off = 0;
-    layout_params(ctx, Lf, (unsigned char *)ctx->net_buf, ctx->h_stage, off, ctx->nf);
-    layout_params(ctx, Ld, (unsigned char *)ctx->net_buf, ctx->h_stage, off, ctx->nd);
+    layout_params(ctx, Lf, (unsigned char *)ctx->net_buf, ctx->h_stage, off, ctx->nf, &ctx->prop32);
+    layout_params(ctx, Ld, (unsigned char *)ctx->net_buf, ctx->h_stage, off, ctx->nd, &ctx->prop64);
+    ctx->net_bytes = bytes;
     for (int k = 1; k + 1 < ctx->K; ++k) ctx->nd.Wsf[k] = ctx->nf.Ws[k];
     std::memcpy(ctx->h_stage + off, ctx->C.data(), ctx->C.size() * sizeof(float));
     ctx->dC = reinterpret_cast<const float *>((unsigned char *)ctx->net_buf + off);
@@ -1101,7 +1177,7 @@ int prepare_device(slr_ctx *ctx) {
         ctx->adj_smem = 0;
         ctx->adj_gmem = true;
         ctx->adj_grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)2 * ctx->sm_count, ((size_t)4 << 30) / box));
-        ctx->dev_dirty = false;
+        ctx->dev_dirty = ctx->net_dirty = false;
         return SLR_OK;
     }
     TileChoice best = c32[0];
@@ -1163,6 +1239,7 @@ int prepare_device(slr_ctx *ctx) {
         ctx->tc_ok = false;
     }
     ctx->dev_dirty = false;
+    ctx->net_dirty = ctx->tc_ok;   // (the tensor-core tile's images hold the property's rows: built anew)
     return SLR_OK;
 }
 
@@ -1451,7 +1528,7 @@ int slr_set_options(slr_ctx *ctx, const slr_options *opt) {
     if (opt->relax_mode != ctx->opt.relax_mode || opt->precision != ctx->opt.precision ||
         opt->tile_boxes != ctx->opt.tile_boxes || opt->tile_threads != ctx->opt.tile_threads ||
         opt->wide != ctx->opt.wide || opt->recheck_cluster != ctx->opt.recheck_cluster)
-        ctx->dev_dirty = true;
+        ctx->dev_dirty = ctx->net_dirty = true;
     ctx->opt = *opt;
     return SLR_OK;
 }
@@ -1478,7 +1555,7 @@ int slr_load_network(slr_ctx *ctx, int K, const int32_t *widths, const float *co
     ctx->b.swap(bv);
     ctx->act.clear();
     ctx->has_net = true;
-    ctx->dev_dirty = true;
+    ctx->dev_dirty = ctx->net_dirty = true;
     ctx->leaves_valid = false;
     return SLR_OK;
 }
@@ -1507,7 +1584,7 @@ int slr_set_activations(slr_ctx *ctx, int n, const int32_t *act) {
         if (act[k] != SLR_ACT_RELU && act[k] != SLR_ACT_TANH && act[k] != SLR_ACT_SIGMOID)
             return fail(ctx, SLR_EINVAL, "activation %d of hidden layer %d unknown", act[k], k);
     ctx->act.assign(act, act + n);
-    ctx->dev_dirty = true;
+    ctx->dev_dirty = ctx->net_dirty = true;
     ctx->leaves_valid = false;
     return SLR_OK;
 }
