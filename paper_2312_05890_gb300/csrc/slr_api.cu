@@ -137,6 +137,8 @@ struct slr_ctx {
     int wide_cols = 0;                    // columns of a box's state: d, padded to its tiles there
     const float *w0b = nullptr;           // layer 1 in the layer kernel's state layout of one box
     const unsigned char *w_img[slr::kMaxLayers] = {};   // its weight pieces per layer
+    unsigned char *wt_img[slr::kMaxLayers] = {};        // and the transposed ones (the adjoint's backward products)
+    bool wt_img_stale = true;             // packed at the first adjoint of a network and property
     int w_Kpad[slr::kMaxLayers] = {};
     // transposed pieces (W_k^T, |W_k|^T) for the adjoint's backward products
     const float *wt_hi[slr::kMaxLayers] = {}, *wt_lo[slr::kMaxLayers] = {};
@@ -653,6 +655,12 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
         offs_l[k] = total;
         total += align_up(slr::wide_layer_img_bytes(nf.n[k], nf.n[k + 1]));
     }
+    std::vector<size_t> offs_lt(K, 0);
+    for (int k = 1; k < K && ctx->wide_layers; ++k) {
+        offs_lt[k] = total;
+        total += align_up(slr::wide_layer_img_bytes(nf.n[k + 1], nf.n[k]));
+    }
+    ctx->wt_img_stale = true;
     if (ctx->wide_img) cudaFree(ctx->wide_img);
     ctx->wide_img = nullptr;
     {
@@ -692,6 +700,7 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
             ctx->wt_lo[k] = (const float *)(bt + oneT);
             ctx->wta_hi[k] = (const float *)(bt + 2 * oneT);
             ctx->wta_lo[k] = (const float *)(bt + 3 * oneT);
+            ctx->wt_img[k] = (unsigned char *)ctx->wide_img + offs_lt[k];
             if (k + 1 < K && ctx->wide_layers) {
                 unsigned char *img = (unsigned char *)ctx->wide_img + offs_l[k];
                 CK(ctx, slr::launch_wide_pack(ctx->w_hi[k], ctx->w_lo[k], ctx->wa_hi[k], ctx->wa_lo[k],
@@ -895,6 +904,10 @@ int run_wide_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int64_t *launches) {
         n = std::min<int64_t>(n, (int64_t)c);
     }
     if (n <= 0) return SLR_OK;
+    if (!ctx->status) {
+        CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
+        CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
+    }
     // chunk: the boxes whose state fits about 6 GB
     const size_t eq = (size_t)Q * np;
     const size_t per_box = sizeof(float) * (eq * (size_t)(2 * (K - 1) - 1 + 6) + 5 * (size_t)(K - 1) * np +
@@ -925,6 +938,29 @@ int run_wide_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int64_t *launches) {
     float *gC = take((size_t)bc * eq), *gR = take((size_t)bc * eq);
     const int64_t sstride = bc * np;
     float *sc = take((size_t)5 * (K - 1) * sstride);
+    if (ctx->wide_layers && ctx->wt_img_stale) {
+        for (int k = 1; k < K; ++k)
+            CK(ctx, slr::launch_wide_pack(ctx->wt_hi[k], ctx->wt_lo[k], ctx->wta_hi[k], ctx->wta_lo[k], ctx->wt_Kpad[k],
+                                          nf.n[k + 1], nf.n[k], ctx->wt_img[k], ctx->stream));
+        ctx->wt_img_stale = false;
+    }
+    // (oc, orr) = (W c, |W| r) over nb boxes of Q columns, W with the given pieces
+    auto product = [&](const unsigned char *img, const slr::WideGemmArgs &ga, int nb) -> cudaError_t {
+        if (!ctx->wide_layers) return slr::launch_wide_gemm(ga, 2, ctx->stream);
+        slr::WideLayer g{};
+        g.Aimg = img;
+        g.Cin = ga.g[0].B;
+        g.Rin = ga.g[1].B;
+        g.Cout = ga.g[0].D;
+        g.Rout = ga.g[1].D;
+        g.nb = nb;
+        g.d = Q;
+        g.NP = np;
+        g.n_in = ga.g[0].K;
+        g.n_out = ga.g[0].M;
+        g.status = ctx->status;
+        return slr::launch_wide_product(g, sms, ctx->stream);
+    };
     for (int64_t pos0 = 0; pos0 < n; pos0 += bc) {
         const int nb = (int)std::min<int64_t>(bc, n - pos0);
         CK(ctx, slr::launch_wadj_box(a.src, pos0, nb, d, m, r, sms, ctx->stream));
@@ -950,7 +986,7 @@ int run_wide_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int64_t *launches) {
                                     nb * Q, np, np};
             ga.g[1] = slr::WideGemm{ctx->wa_hi[k], ctx->wa_lo[k], Pr, orr, nf.n[k + 1], nf.n[k], ctx->w_Kpad[k],
                                     nb * Q, np, np};
-            CK(ctx, slr::launch_wide_gemm(ga, 2, ctx->stream));
+            CK(ctx, product(ctx->w_img[k], ga, nb));
             *launches += 2;
         }
         CK(ctx, slr::launch_wadj_rows(a, pos0, nb, np, Cf, Rf, nf.b[K - 1], gC, gR, ctx->stream));
@@ -962,7 +998,7 @@ int run_wide_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int64_t *launches) {
                                     nb * Q, np, np};
             ga.g[1] = slr::WideGemm{ctx->wta_hi[k], ctx->wta_lo[k], gR, Pr, nf.n[k], nf.n[k + 1], ctx->wt_Kpad[k],
                                     nb * Q, np, np};
-            CK(ctx, slr::launch_wide_gemm(ga, 2, ctx->stream));
+            CK(ctx, product(ctx->wt_img[k], ga, nb));
             const float *sck = sc + (size_t)(k - 1) * 5 * sstride;
             CK(ctx, slr::launch_wadj_bwd(a, k, pos0, nb, np, Cl[k], Rl[k], sck, sstride, Pc, Pr, gC,
                                          k > 1 ? gR : nullptr, ctx->stream));
@@ -1109,6 +1145,7 @@ int new_property(slr_ctx *ctx) {
         fill_pieces(Lf, K - 1, n_in, n_out, ctx->w_Kpad[K - 1], ctx->wt_Kpad[K - 1], pf, pb);
         CK(ctx, cudaMemcpyAsync((void *)ctx->w_hi[K - 1], pf, fwd, cudaMemcpyHostToDevice, ctx->stream));
         CK(ctx, cudaMemcpyAsync((void *)ctx->wt_hi[K - 1], pb, bwd, cudaMemcpyHostToDevice, ctx->stream));
+        ctx->wt_img_stale = true;
     }
     CK(ctx, cudaStreamSynchronize(ctx->stream));
     ctx->dev_dirty = false;

@@ -200,7 +200,9 @@ size_t wide_layer_img_bytes(int n_in, int n_out);
 int wide_rows_stride(int R);
 cudaError_t launch_wide_pack(const float *hi, const float *lo, const float *ahi, const float *alo, int ld, int n_in,
                              int n_out, void *out, cudaStream_t s);
-cudaError_t launch_wide_layer(WideLayer G, int sms, cudaStream_t s);
+cudaError_t launch_wide_layer(const WideLayer &G, int sms, cudaStream_t s);
+// The two products alone on states [b][d][NP] (plan, part, W0b and rr unused).
+cudaError_t launch_wide_product(const WideLayer &G, int sms, cudaStream_t s);
 cudaError_t launch_wide_plan1(const NetParams<float> &net, const float *W0t, int nb, int NP, const float *mh,
                               const float *ml, const float *rr, float *plan, float *S3, float *Ch, float *Cl,
                               const float *alpha, int64_t alpha_ld, int64_t base, cudaStream_t s);

@@ -790,6 +790,9 @@ cudaError_t launch_wide_rows_product(const float *Wt, int n_in, int R, const flo
     } else if (R <= 8) {
         wide_rows_product_kernel<8><<<grid, 256, (size_t)n_in * 8 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D, ldd,
                                                                                        ncols, abs_w ? 1 : 0);
+    } else if (R <= 12) {
+        wide_rows_product_kernel<12><<<grid, 256, (size_t)n_in * 12 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D,
+                                                                                         ldd, ncols, abs_w ? 1 : 0);
     } else if (R <= 16) {
         wide_rows_product_kernel<16><<<grid, 256, (size_t)n_in * 16 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D,
                                                                                          ldd, ncols, abs_w ? 1 : 0);

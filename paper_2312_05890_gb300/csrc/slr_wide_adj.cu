@@ -19,8 +19,10 @@
 //
 // Layout as the sound wide path: [box][column][neuron], columns 0..d-1 the
 // coefficients of the normalised inputs and column d the constant, neuron
-// row stride NP.  Row kernels: a block is 32 neurons (threadIdx.x) of one box
-// (blockIdx.y) with the columns split over 16 slices (threadIdx.y).
+// row stride NP.  Row kernels: a block is 128 neurons of one box (blockIdx.y),
+// four neighbouring ones per thread (threadIdx.x; a float4 of every column, 512
+// bytes per warp), with the columns split over 16 slices (threadIdx.y) whose
+// sums are added in slice order.  DRAM bounds them: ADJ_NOTE
 #include <algorithm>
 
 #include "slr_adj_common.cuh"
@@ -35,6 +37,24 @@ constexpr int kAX = 32, kAY = 16;
 
 __device__ __forceinline__ size_t at(int64_t b, int Q, int c, int NP, int p) {
     return ((size_t)b * Q + c) * NP + p;
+}
+
+constexpr int kA4Rows = 4 * kAX;   // neurons of a row kernel's block
+
+__device__ __forceinline__ void ld4(const float *p, float (&v)[4]) {
+    const float4 t = *reinterpret_cast<const float4 *>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+    v[2] = t.z;
+    v[3] = t.w;
+}
+// the first `n` of four values (n >= 4: all; the others lie past the layer's width)
+__device__ __forceinline__ void st4(float *p, const float (&v)[4], int n) {
+    if (n >= 4) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+        return;
+    }
+    for (int u = 0; u < n; ++u) p[u] = v[u];
 }
 
 }  // namespace
@@ -77,7 +97,9 @@ wadj_layer1_kernel(const NetParams<float> net, const float *W0t, int NP, const f
     const float *mb = m + b * d, *rb = r + b * d;
     for (int j = threadIdx.y; j < d; j += kAY) C[at(b, Q, j, NP, p)] = W0t[(size_t)j * n1 + p] * rb[j];
     if (threadIdx.y == 0) {
+        // (one chain: sixteen loads of it in flight)
         float v = __ldg(net.b[0] + p);
+#pragma unroll 16
         for (int i = 0; i < d; ++i) v = fmaf(W0t[(size_t)i * n1 + p], mb[i], v);
         C[at(b, Q, d, NP, p)] = v;
     }
@@ -89,34 +111,47 @@ wadj_layer1_kernel(const NetParams<float> net, const float *W0t, int NP, const f
 __global__ void __launch_bounds__(kAX * kAY)
 wadj_fwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, float *C, const float *R, const float *bias,
                 float *sc, int64_t sstride, float *Pc, float *Pr) {
-    __shared__ float psu[kAY][kAX], psl[kAY][kAX];
-    __shared__ float sp[5][kAX];
+    __shared__ float psu[kAY][kA4Rows], psl[kAY][kA4Rows];
+    __shared__ float sp[5][kA4Rows];
     const NetParams<float> &net = a.net;
     const int d = net.d, Q = d + 1, n = net.n[layer];
     const int lane = threadIdx.x, sl = threadIdx.y;
-    const int p = blockIdx.x * kAX + lane;
+    const int pb = blockIdx.x * kA4Rows, p0 = pb + 4 * lane;
     const int64_t b = blockIdx.y;
-    const bool live = p < n;
-    float su = 0.f, sv = 0.f;
-    if (live) {
-        if (sl == 0 && bias != nullptr) C[at(b, Q, d, NP, p)] += __ldg(bias + p);
+    const bool any = p0 < n;
+    float su[4] = {0.f, 0.f, 0.f, 0.f}, sv[4] = {0.f, 0.f, 0.f, 0.f};
+    if (any) {
+#pragma unroll 4
         for (int c = sl; c < d; c += kAY) {
-            const float cv = C[at(b, Q, c, NP, p)];
-            const float rv = R != nullptr ? R[at(b, Q, c, NP, p)] : 0.f;
-            su += fabsf(cv + rv);
-            sv += fabsf(cv - rv);
+            float cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f};
+            ld4(C + at(b, Q, c, NP, p0), cv);
+            if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                su[u] += fabsf(cv[u] + rv[u]);
+                sv[u] += fabsf(cv[u] - rv[u]);
+            }
         }
     }
-    psu[sl][lane] = su;
-    psl[sl][lane] = sv;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        psu[sl][4 * lane + u] = su[u];
+        psl[sl][4 * lane + u] = sv[u];
+    }
     __syncthreads();
-    if (sl == 0 && live) {
+    // the first four slices: one row per thread
+    const int row = sl * kAX + lane, p = pb + row;
+    if (sl < kA4Rows / kAX && p < n) {
         float tu = 0.f, tl = 0.f;
         for (int y = 0; y < kAY; ++y) {
-            tu += psu[y][lane];
-            tl += psl[y][lane];
+            tu += psu[y][row];
+            tl += psl[y][row];
         }
-        const float cd = C[at(b, Q, d, NP, p)];
+        float cd = C[at(b, Q, d, NP, p)];
+        if (bias != nullptr) {
+            cd += __ldg(bias + p);
+            C[at(b, Q, d, NP, p)] = cd;
+        }
         const float rd = R != nullptr ? R[at(b, Q, d, NP, p)] : 0.f;
         const float ud = cd + rd, ldv = cd - rd;
         const float ll = ldv - tl, ul = ldv + tl, lu = ud - tu, uu = ud + tu;
@@ -132,35 +167,47 @@ wadj_fwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, float *C, cons
         }
         const float v[5] = {ll, ul, lu, uu, al};
         for (int q = 0; q < 5; ++q) {
-            sp[q][lane] = v[q];
+            sp[q][row] = v[q];
             sc[q * sstride + b * NP + p] = v[q];
         }
     }
     __syncthreads();
-    if (!live) return;
-    const float ll = sp[0][lane], ul = sp[1][lane], lu = sp[2][lane], uu = sp[3][lane], al = sp[4][lane];
+    if (!any) return;
+    float ll[4], ul[4], lu[4], uu[4], al[4];
+    ld4(&sp[0][4 * lane], ll);
+    ld4(&sp[1][4 * lane], ul);
+    ld4(&sp[2][4 * lane], lu);
+    ld4(&sp[3][4 * lane], uu);
+    ld4(&sp[4][4 * lane], al);
+#pragma unroll 4
     for (int c = sl; c < Q; c += kAY) {
-        const float cv = C[at(b, Q, c, NP, p)];
-        const float rv = R != nullptr ? R[at(b, Q, c, NP, p)] : 0.f;
-        const float u = cv + rv, l = cv - rv;
-        float uh, lh;
-        if (ll >= 0.f) {
-            uh = u;
-            lh = l;
-        } else if (uu <= 0.f) {
-            uh = 0.f;
-            lh = 0.f;
-        } else {
-            if (lu >= 0.f) {
+        float cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f}, oc[4], orr[4];
+        ld4(C + at(b, Q, c, NP, p0), cv);
+        if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float u = cv[k] + rv[k], l = cv[k] - rv[k];
+            float uh, lh;
+            if (ll[k] >= 0.f) {
                 uh = u;
+                lh = l;
+            } else if (uu[k] <= 0.f) {
+                uh = 0.f;
+                lh = 0.f;
             } else {
-                const float sg = uu / (uu - lu);
-                uh = sg * (c == d ? u - lu : u);
+                if (lu[k] >= 0.f) {
+                    uh = u;
+                } else {
+                    const float sg = uu[k] / (uu[k] - lu[k]);
+                    uh = __fmul_rn(sg, c == d ? u - lu[k] : u);
+                }
+                lh = ul[k] > 0.f ? __fmul_rn(al[k], l) : 0.f;
             }
-            lh = ul > 0.f ? al * l : 0.f;
+            oc[k] = 0.5f * __fadd_rn(uh, lh);
+            orr[k] = 0.5f * __fsub_rn(uh, lh);
         }
-        Pc[at(b, Q, c, NP, p)] = 0.5f * (uh + lh);
-        Pr[at(b, Q, c, NP, p)] = 0.5f * (uh - lh);
+        st4(Pc + at(b, Q, c, NP, p0), oc, n - p0);
+        st4(Pr + at(b, Q, c, NP, p0), orr, n - p0);
     }
 }
 
@@ -229,35 +276,46 @@ wadj_rows_kernel(const AdjArgs a, int64_t pos0, int NP, const float *C, const fl
 // adjoints (gPc, gPr) of the products' inputs to those of the pre-activation
 // equations, written as (gC, gR) = (gU + gL, gU - gL) (gR null at layer 1,
 // where U = L); the slope gradient and its projected-Adam step.
-__global__ void __launch_bounds__(kAX * kAY)
+__global__ void __launch_bounds__(kAX * kAY, 2)
 wadj_bwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, const float *C, const float *R, const float *sc,
                 int64_t sstride, const float *gPc, const float *gPr, float *gC, float *gR) {
-    __shared__ float ps[kAY][kAX], pa[kAY][kAX];
-    __shared__ float sp[8][kAX];
+    __shared__ float ps[kAY][kA4Rows], pa[kAY][kA4Rows];
+    __shared__ float sp[8][kA4Rows];
     const NetParams<float> &net = a.net;
     const int d = net.d, Q = d + 1, n = net.n[layer];
     const int lane = threadIdx.x, sl = threadIdx.y;
-    const int p = blockIdx.x * kAX + lane;
+    const int pb = blockIdx.x * kA4Rows, p0 = pb + 4 * lane;
     const int64_t b = blockIdx.y;
-    const bool live = p < n;
-    float gs = 0.f, ga = 0.f;
-    if (live) {
+    const bool any = p0 < n;
+    float gs[4] = {0.f, 0.f, 0.f, 0.f}, ga[4] = {0.f, 0.f, 0.f, 0.f};
+    if (any) {
+#pragma unroll 2
         for (int c = sl; c < Q; c += kAY) {
-            const float gc = gPc[at(b, Q, c, NP, p)], gr = gPr[at(b, Q, c, NP, p)];
-            const float cv = C[at(b, Q, c, NP, p)];
-            const float rv = R != nullptr ? R[at(b, Q, c, NP, p)] : 0.f;
-            gs = fmaf(0.5f * (gc + gr), cv + rv, gs);
-            ga = fmaf(0.5f * (gc - gr), cv - rv, ga);
+            float gc[4], gr[4], cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f};
+            ld4(gPc + at(b, Q, c, NP, p0), gc);
+            ld4(gPr + at(b, Q, c, NP, p0), gr);
+            ld4(C + at(b, Q, c, NP, p0), cv);
+            if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                gs[u] = fmaf(0.5f * (gc[u] + gr[u]), cv[u] + rv[u], gs[u]);
+                ga[u] = fmaf(0.5f * (gc[u] - gr[u]), cv[u] - rv[u], ga[u]);
+            }
         }
     }
-    ps[sl][lane] = gs;
-    pa[sl][lane] = ga;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        ps[sl][4 * lane + u] = gs[u];
+        pa[sl][4 * lane + u] = ga[u];
+    }
     __syncthreads();
-    if (sl == 0 && live) {
+    // the first four slices: one row per thread
+    const int row = sl * kAX + lane, p = pb + row;
+    if (sl < kA4Rows / kAX && p < n) {
         float g_s = 0.f, g_a = 0.f;
         for (int y = 0; y < kAY; ++y) {
-            g_s += ps[y][lane];
-            g_a += pa[y][lane];
+            g_s += ps[y][row];
+            g_a += pa[y][row];
         }
         const float ll = sc[0 * sstride + b * NP + p], ul = sc[1 * sstride + b * NP + p];
         const float lu = sc[2 * sstride + b * NP + p], uu = sc[3 * sstride + b * NP + p];
@@ -300,35 +358,50 @@ wadj_bwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, const float *C
         if (a.d_alpha != nullptr) a.d_alpha[ai] = g_alpha;
         if (a.adam_t > 0 && a.alpha_mode != kAlphaDefault) a.alpha[ai] = adam_slope(a, ai, al, g_alpha);
         const float v[8] = {kind, chord, sg, du, su, lw, dl, sl2};
-        for (int q = 0; q < 8; ++q) sp[q][lane] = v[q];
+        for (int q = 0; q < 8; ++q) sp[q][row] = v[q];
     }
     __syncthreads();
-    if (!live) return;
-    const float kind = sp[0][lane], chord = sp[1][lane], sg = sp[2][lane], du = sp[3][lane], su = sp[4][lane];
-    const float lw = sp[5][lane], dl = sp[6][lane], sl2 = sp[7][lane];
+    if (!any) return;
+    float kind[4], chord[4], sg[4], du[4], su[4], lw[4], dl[4], sl2[4];
+    ld4(&sp[0][4 * lane], kind);
+    ld4(&sp[1][4 * lane], chord);
+    ld4(&sp[2][4 * lane], sg);
+    ld4(&sp[3][4 * lane], du);
+    ld4(&sp[4][4 * lane], su);
+    ld4(&sp[5][4 * lane], lw);
+    ld4(&sp[6][4 * lane], dl);
+    ld4(&sp[7][4 * lane], sl2);
+#pragma unroll 1
     for (int c = sl; c < Q; c += kAY) {
-        const float gc = gPc[at(b, Q, c, NP, p)], gr = gPr[at(b, Q, c, NP, p)];
-        const float gu = 0.5f * (gc + gr), gl = 0.5f * (gc - gr);
-        float oU, oL;
-        if (kind == 0.f) {
-            oU = gu;
-            oL = gl;
-        } else if (kind == 1.f) {
-            oU = 0.f;
-            oL = 0.f;
-        } else {
-            const float cv = C[at(b, Q, c, NP, p)];
-            const float rv = R != nullptr ? R[at(b, Q, c, NP, p)] : 0.f;
-            if (chord != 0.f) {
-                oU = c < d ? sg * gu + du * sgnf(cv + rv) : sg * gu + su;
-            } else {
+        float gc[4], gr[4], cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f}, oc[4], orr[4];
+        ld4(gPc + at(b, Q, c, NP, p0), gc);
+        ld4(gPr + at(b, Q, c, NP, p0), gr);
+        ld4(C + at(b, Q, c, NP, p0), cv);
+        if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float gu = 0.5f * (gc[k] + gr[k]), gl = 0.5f * (gc[k] - gr[k]);
+            float oU, oL;
+            if (kind[k] == 0.f) {
                 oU = gu;
+                oL = gl;
+            } else if (kind[k] == 1.f) {
+                oU = 0.f;
+                oL = 0.f;
+            } else {
+                if (chord[k] != 0.f) {
+                    oU = c < d ? sg[k] * gu + du[k] * sgnf(cv[k] + rv[k]) : sg[k] * gu + su[k];
+                } else {
+                    oU = gu;
+                }
+                oL = __fmul_rn(lw[k], gl);
+                if (dl[k] != 0.f || sl2[k] != 0.f) oL += c < d ? dl[k] * sgnf(cv[k] - rv[k]) : sl2[k];
             }
-            oL = lw * gl;
-            if (dl != 0.f || sl2 != 0.f) oL += c < d ? dl * sgnf(cv - rv) : sl2;
+            oc[k] = oU + oL;
+            orr[k] = oU - oL;
         }
-        gC[at(b, Q, c, NP, p)] = oU + oL;
-        if (gR != nullptr) gR[at(b, Q, c, NP, p)] = oU - oL;
+        st4(gC + at(b, Q, c, NP, p0), oc, n - p0);
+        if (gR != nullptr) st4(gR + at(b, Q, c, NP, p0), orr, n - p0);
     }
 }
 
@@ -412,8 +485,8 @@ cudaError_t launch_wadj_layer1(const NetParams<float> &net, const float *W0t, in
 
 cudaError_t launch_wadj_fwd(const AdjArgs &a, int layer, int64_t pos0, int nb, int NP, float *C, const float *R,
                             const float *bias, float *sc, int64_t sstride, float *Pc, float *Pr, cudaStream_t s) {
-    wadj_fwd_kernel<<<dim3((a.net.n[layer] + kAX - 1) / kAX, nb), dim3(kAX, kAY), 0, s>>>(a, layer, pos0, NP, C, R,
-                                                                                          bias, sc, sstride, Pc, Pr);
+    wadj_fwd_kernel<<<dim3((a.net.n[layer] + kA4Rows - 1) / kA4Rows, nb), dim3(kAX, kAY), 0, s>>>(
+        a, layer, pos0, NP, C, R, bias, sc, sstride, Pc, Pr);
     return cudaGetLastError();
 }
 
@@ -426,7 +499,7 @@ cudaError_t launch_wadj_rows(const AdjArgs &a, int64_t pos0, int nb, int NP, con
 cudaError_t launch_wadj_bwd(const AdjArgs &a, int layer, int64_t pos0, int nb, int NP, const float *C, const float *R,
                             const float *sc, int64_t sstride, const float *gPc, const float *gPr, float *gC, float *gR,
                             cudaStream_t s) {
-    wadj_bwd_kernel<<<dim3((a.net.n[layer] + kAX - 1) / kAX, nb), dim3(kAX, kAY), 0, s>>>(
+    wadj_bwd_kernel<<<dim3((a.net.n[layer] + kA4Rows - 1) / kA4Rows, nb), dim3(kAX, kAY), 0, s>>>(
         a, layer, pos0, NP, C, R, sc, sstride, gPc, gPr, gC, gR);
     return cudaGetLastError();
 }

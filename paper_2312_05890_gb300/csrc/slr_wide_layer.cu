@@ -130,6 +130,9 @@ __device__ __forceinline__ void relax_pair(float pp, float qq, float c0, float r
 
 }  // namespace
 
+// kPlain: the two products alone, D_C = W C, D_R = |W| R on states [box][column][NP]
+// (the wide adjoint): no relaxation, no bound sums.
+template <bool kPlain>
 __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLayer G) {
     extern __shared__ __align__(1024) unsigned char smem_l[];
     const int NA = G.na, NC = G.NC, bimg = b_img(NC), bstep = b_step(NC), bstage = b_stage(NC);
@@ -166,7 +169,11 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
     const uint32_t tmem = *tslot;
 
     const int nst = G.nst;
-    const size_t tile = (size_t)NC * G.NP;        // floats of one tile of the state
+    // the state of column cc of tile t of box b, inputs or rows 16 k ..: from
+    // ((b boxes) + t tiles) + cc cs + k ks
+    const size_t tile = (size_t)NC * G.NP;
+    const size_t boxs = kPlain ? (size_t)G.d * G.NP : G.ntile * tile;
+    const int cs = kPlain ? G.NP : kLK, ks = kPlain ? kLK : NC * kLK;
     const int per_box = G.ntile * G.mt;
     const int items = G.nb * per_box;             // item = (box, column tile, row tile), row tile fastest
     const int mine = (items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;   // (the grid has at most `items` CTAs)
@@ -217,24 +224,24 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
                 }
                 const int j0 = t * NC + 16 * ch;
                 if (p < G.n_out) {
-                    const size_t o = ((size_t)b * G.ntile + t) * tile + ((size_t)(p / kLK) * NC + 16 * ch) * kLK + p % kLK;
+                    const size_t o = b * boxs + t * tile + (size_t)(p / kLK) * ks + (size_t)(16 * ch) * cs + p % kLK;
                     float *co = G.Cout + o, *ro = G.Rout + o;
                     if (j0 + 16 <= G.d) {
 #pragma unroll
                         for (int e = 0; e < 16; ++e) {
                             const float cv = __uint_as_float(c[e]), rv = __uint_as_float(r[e]);
-                            bd.add(cv, rv);
-                            co[e * kLK] = cv;
-                            ro[e * kLK] = rv;
+                            if (!kPlain) bd.add(cv, rv);
+                            co[e * cs] = cv;
+                            ro[e * cs] = rv;
                         }
                     } else {
 #pragma unroll
                         for (int e = 0; e < 16; ++e) {
                             if (j0 + e < G.d) {
                                 const float cv = __uint_as_float(c[e]), rv = __uint_as_float(r[e]);
-                                bd.add(cv, rv);
-                                co[e * kLK] = cv;
-                                ro[e * kLK] = rv;
+                                if (!kPlain) bd.add(cv, rv);
+                                co[e * cs] = cv;
+                                ro[e * cs] = rv;
                             }
                         }
                     }
@@ -245,7 +252,7 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(tempty));
             }
-            if (p < G.n_out) {
+            if (!kPlain && p < G.n_out) {
                 float *q = G.part + (((size_t)b * G.ntile + t) * 3 + slice) * 4 * G.NP + p;
                 q[0] = bd.SU;
                 q[G.NP] = bd.SL;
@@ -259,7 +266,7 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
         // that a load of a warp reads 64-byte runs of eight columns ----
         const int q = lane & 3;
         const int col = warp * 8 + (lane >> 2);
-        const bool gen = G.Cin == nullptr;
+        const bool gen = !kPlain && G.Cin == nullptr;
         // The loads are unconditional (columns past the tile's end and stages past
         // the last one repeat valid addresses and are not used): a load under a
         // condition is merged with the value it replaces, which waits for it.
@@ -272,9 +279,9 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int cc = min(col + 8 * kLWork * u, NC - 1), j = min(t * NC + cc, G.d - 1);
-                const size_t o = (size_t)(j - t * NC) * kLK + 4 * q;
-                cp[u] = gen ? G.W0b + (size_t)t * tile + o : G.Cin + ((size_t)b * G.ntile + t) * tile + o;
-                rp[u] = gen ? cp[u] : G.Rin + ((size_t)b * G.ntile + t) * tile + o;
+                const size_t o = t * tile + (size_t)(j - t * NC) * cs + 4 * q;
+                cp[u] = gen ? G.W0b + o : G.Cin + b * boxs + o;
+                rp[u] = gen ? cp[u] : G.Rin + b * boxs + o;
                 rj[u] = gen ? G.rr[(size_t)b * G.d + j] : 0.f;
             }
         };
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
         auto load = [&](Raw &v) {
             // (inputs from n_in to the end of the last stage lie within the tile
             // and their plan is zero)
-            const size_t o = (size_t)lst * NC * kLK;
+            const size_t o = (size_t)lst * ks;
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 v.c[u] = *reinterpret_cast<const float4 *>(cp[u] + o);
@@ -299,6 +306,7 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
         // warp, so one stage ahead is enough
         float4 pp, qq;
         auto load_plan = [&](int use, int st) {
+            if (kPlain) return;
             const float *pl = G.plan + (size_t)((blockIdx.x + min(use, mine - 1) * gridDim.x) / per_box) * 2 * G.NP + st * kLK + 4 * q;
             pp = *reinterpret_cast<const float4 *>(pl);
             qq = *reinterpret_cast<const float4 *>(pl + G.NP);
@@ -323,8 +331,15 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
                 const float r0[4] = {v.r[u].x, v.r[u].y, v.r[u].z, v.r[u].w};
                 float c[4], r[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    relax_pair(pv[e], qv[e], gen ? __fmul_rn(c0[e], v.rj[u]) : c0[e], gen ? 0.f : r0[e], c[e], r[e]);
+                for (int e = 0; e < 4; ++e) {
+                    if (kPlain) {
+                        const bool in = st * kLK + 4 * q + e < G.n_in;
+                        c[e] = in ? c0[e] : 0.f;
+                        r[e] = in ? r0[e] : 0.f;
+                    } else {
+                        relax_pair(pv[e], qv[e], gen ? __fmul_rn(c0[e], v.rj[u]) : c0[e], gen ? 0.f : r0[e], c[e], r[e]);
+                    }
+                }
                 if (cc < NC) {
                     unsigned char *o = to + (cc >> 3) * kLSboB + (cc & 7) * 16;
                     split4(c, o, o + bimg);
@@ -870,7 +885,8 @@ cudaError_t launch_wide_pack(const float *hi, const float *lo, const float *ahi,
     return cudaGetLastError();
 }
 
-cudaError_t launch_wide_layer(WideLayer G, int sms, cudaStream_t s) {
+template <bool kPlain>
+static cudaError_t launch_layer(WideLayer G, int sms, cudaStream_t s) {
     G.mt = (G.n_out + kLRows - 1) / kLRows;
     G.nst = (G.n_in + kLK - 1) / kLK;
     wide_layer_tiles(G.d, G.ntile, G.NC);
@@ -879,11 +895,15 @@ cudaError_t launch_wide_layer(WideLayer G, int sms, cudaStream_t s) {
     if (items > INT32_MAX) return cudaErrorInvalidValue;
     G.na = a_stages(G.NC);
     const int smem = G.na * kLA + kBStages * b_stage(G.NC) + kLBar;
-    cudaError_t e = cudaFuncSetAttribute(wide_layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(wide_layer_kernel<kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    wide_layer_kernel<<<(int)std::min<int64_t>(items, sms), kLThreads, smem, s>>>(G);
+    wide_layer_kernel<kPlain><<<(int)std::min<int64_t>(items, sms), kLThreads, smem, s>>>(G);
     return cudaGetLastError();
 }
+
+cudaError_t launch_wide_layer(const WideLayer &G, int sms, cudaStream_t s) { return launch_layer<false>(G, sms, s); }
+
+cudaError_t launch_wide_product(const WideLayer &G, int sms, cudaStream_t s) { return launch_layer<true>(G, sms, s); }
 
 cudaError_t launch_wide_plan1(const NetParams<float> &net, const float *W0t, int nb, int NP, const float *mh,
                               const float *ml, const float *rr, float *plan, float *S3, float *Ch, float *Cl,

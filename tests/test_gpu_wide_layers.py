@@ -10,7 +10,7 @@ import oracle
 from workloads import generators as gen
 
 from .gpu_common import BOUND_RTOL, bound_errors, random_sub_boxes
-from .test_gpu_alpha import _split_alpha_batch
+from .test_gpu_alpha import _close, _split_alpha, _split_alpha_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +89,37 @@ def test_more_boxes_than_a_chunk(pkg):
         rl, rh, _ = c.bounds(lo, hi)
         part = c.bounds(lo[1300:], hi[1300:])
     assert np.array_equal(rl[1300:], part[0]) and np.array_equal(rh[1300:], part[1])
+
+
+@pytest.mark.parametrize("d,hidden,R,n", [(64, [8, 8], 1, 1), (223, [40], 3, 2), (224, [129, 33], 5, 3),
+                                          (100, [60, 61, 62], 13, 4), (300, [256, 130], 9, 2)])
+@pytest.mark.parametrize("free", [True, False])
+def test_adjoint(pkg, d, hidden, R, n, free):
+    """The adjoint's products on the same kernel (d + 1 columns), forward and through the
+    transposed weights, against central differences at sampled coordinates."""
+    p = _problem(d, hidden, R)
+    rng = np.random.default_rng(d)
+    lo, hi = random_sub_boxes(p, n, seed=n)
+    H = sum(hidden)
+    g_lo, g_hi = (rng.normal(size=(n, R)).astype(np.float32) for _ in range(2))
+    A = rng.uniform(0.05, 0.95, size=(n, H)).astype(np.float32) if free else None
+    a_idx = rng.choice(H, size=min(H, 30), replace=False)
+    x_idx = rng.choice(d, size=20, replace=False)
+    with pkg.Counter(0) as c:
+        c.set_problem(p)
+        c.set_options(wide=1)
+        whole = c.margin_backward(lo, hi, g_lo, g_hi, alpha=A)
+        for i in range(n):
+            one = c.margin_backward(lo[i:i + 1], hi[i:i + 1], g_lo[i:i + 1], g_hi[i:i + 1],
+                                    alpha=None if A is None else A[i:i + 1])
+            for key in whole:
+                assert np.array_equal(whole[key][i:i + 1], one[key]), key
+    for i in (0, n - 1):
+        fd = oracle.fd_gradients(p.net, lo[i], hi[i], p.prop,
+                                 _split_alpha(p.net, A[i].astype(np.float64)) if free else None,
+                                 g_hi[i].astype(np.float64), g_lo[i].astype(np.float64), h=1e-4, w_idx={},
+                                 alpha_idx=a_idx if free else None, box_idx=x_idx)
+        checks = [("d_lo", fd["lo"]), ("d_hi", fd["hi"])] + ([("d_alpha", np.concatenate(fd["alpha"]))] if free else [])
+        for key, want in checks:
+            ok, e = _close(whole[key][i], want, 2e-3)
+            assert ok, (key, i, e)
