@@ -254,8 +254,8 @@ adj_warp_kernel(const AdjArgs a, const AdjWarpPlan pl, float *chk) {
                     int c;
                     code_dim(src, src.codes[idx], lane, kk, c);
                     const double w = src.root_w[lane];
-                    r64 = ldexp(w, -(c + 1));
-                    m64 = src.root_lo[lane] + w * ldexp((double)(2 * kk + 1), -(c + 1));
+                    r64 = w * pow2_neg(c + 1);
+                    m64 = src.root_lo[lane] + w * ((double)(2 * kk + 1) * pow2_neg(c + 1));
                 } else {
                     const double blo = (double)src.lo[idx * d + lane];
                     const double bhi = (double)src.hi[idx * d + lane];

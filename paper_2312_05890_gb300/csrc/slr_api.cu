@@ -568,9 +568,16 @@ int autotune(slr_ctx *ctx, const std::vector<TileChoice> &cands, TileChoice &bes
         CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
     }
     o.status = ctx->status;
-    float best_ms = 1e30f;
+    // each choice on as many boxes as fill whole rounds of its grid (where a
+    // round fits): a partly filled last round would decide between tiles that
+    // differ by less (16 and 20 boxes of a 5-6x50-5 network: the larger one is
+    // 14 % faster on long runs and took 3 rounds of 16384 boxes against 4)
+    float best_ms = 1e30f;   // per box
     for (const TileChoice &c : cands) {
-        const int grid = (int)std::min<int64_t>((n + c.T - 1) / c.T, (int64_t)c.blocks * ctx->sm_count);
+        const int64_t round = (int64_t)c.T * c.blocks * ctx->sm_count;
+        const int64_t nc = n >= round ? n / round * round : n;
+        src.n_explicit = src.cap = nc;
+        const int grid = (int)std::min<int64_t>((nc + c.T - 1) / c.T, (int64_t)c.blocks * ctx->sm_count);
         float ms = 0.f;
         for (int rep = 0; rep < 3; ++rep) {
             CK(ctx, cudaEventRecord(ctx->ev0, ctx->stream));
@@ -579,7 +586,7 @@ int autotune(slr_ctx *ctx, const std::vector<TileChoice> &cands, TileChoice &bes
             CK(ctx, cudaEventSynchronize(ctx->ev1));
             float t = 0.f;
             cudaEventElapsedTime(&t, ctx->ev0, ctx->ev1);
-            if (rep > 0) ms += t;     // the first run warms the caches
+            if (rep > 0) ms += t / (float)nc;     // the first run warms the caches
         }
         if (ms < best_ms) {
             best_ms = ms;
@@ -1032,6 +1039,12 @@ int run_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int grid, int64_t *launches
     return SLR_OK;
 }
 
+// CTAs for a level of at most 2^t boxes (a launch that finds nothing to do ends
+// sooner with one CTA than with one per SM).
+int level_grid(int grid, int T, int t) {
+    return t > 24 ? grid : (int)std::min<int64_t>(grid, (((int64_t)1 << t) + T - 1) / T);
+}
+
 // FP64 re-check of a list of boxes at level t: on clusters where chosen (pass
 // 1); else, with recheck_pairs, the float-float stage (pass 2), after which a
 // tile that still holds boxes depending on E is bounded again with plain FP64
@@ -1042,8 +1055,8 @@ cudaError_t launch_recheck(slr_ctx *ctx, const slr::BoxSource &src, const slr::E
     slr::EvalOutputs o = out;
     const bool pairs = ctx->opt.recheck_pairs && ctx->pairs_fit;
     if (pairs) o.near_count = &ctx->ctr->near3_n[t];
-    return slr::launch_eval_f64(ctx->T64, ctx->NT64, ctx->grid64, ctx->smem64, ctx->stream, ctx->nd, src, o,
-                                pairs ? 2 : 1);
+    return slr::launch_eval_f64(ctx->T64, ctx->NT64, level_grid(ctx->grid64, ctx->T64, t), ctx->smem64, ctx->stream,
+                                ctx->nd, src, o, pairs ? 2 : 1);
 }
 
 // FP64 re-check: short lists, so the smallest tiles spread them over the
@@ -1413,7 +1426,7 @@ void slr_internal_level_tile(const slr_ctx *ctx, int t, int *T, int *NT, int *gr
     const TileChoice c = level_tile(ctx, t);
     *T = c.T;
     *NT = c.NT;
-    *grid = c.blocks * ctx->sm_count;
+    *grid = level_grid(c.blocks * ctx->sm_count, c.T, t);
     *smem = c.smem;
 }
 
@@ -1863,8 +1876,8 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
             }
         } else {
         const TileChoice tile = level_tile(ctx, t);
-        CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, tile.blocks * ctx->sm_count, tile.smem, ctx->stream, ctx->nf, src,
-                                     o, 0));
+        CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, level_grid(tile.blocks * ctx->sm_count, tile.T, t), tile.smem,
+                                     ctx->stream, ctx->nf, src, o, 0));
         CK(ctx, mark(t, 1));
         ++launches;
         if (recheck) {
@@ -2417,11 +2430,15 @@ int slr_bounds(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi
         CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
     }
     o.status = ctx->status;
-    CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned int), ctx->stream));
+    // only the tensor-core paths report through the status word here (the FP32
+    // tile writes it when a re-check list overflows, and bounds have none)
+    const bool tc = ctx->opt.precision == SLR_PREC_TC_TF32 && ctx->tc_ok && alpha == nullptr;
+    const bool reports = ctx->wide || tc;
+    if (reports) CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned int), ctx->stream));
     if (ctx->wide) {
         int64_t launches = 0;
         if ((rc = run_wide(ctx, src, n, o, &launches))) return rc;
-    } else if (ctx->opt.precision == SLR_PREC_TC_TF32 && ctx->tc_ok && alpha == nullptr) {
+    } else if (tc) {
         const int64_t tiles = (n + ctx->T_tc - 1) / ctx->T_tc;
         const int grid = (int)std::min<int64_t>(tiles, ctx->grid_tc);
         CK(ctx, slr::launch_eval_tc(ctx->T_tc, grid, ctx->smem_tc, ctx->stream, ctx->nf, ctx->tcp, src, o, 0));
@@ -2439,9 +2456,10 @@ int slr_bounds(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi
             CK(ctx, cudaMemcpyAsync(row_err, dre, (size_t)n * R * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
         if (cls) CK(ctx, cudaMemcpyAsync(cls, dcls, (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
     }
-    CK(ctx, cudaMemcpyAsync(ctx->h_status, ctx->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
+    if (reports)
+        CK(ctx, cudaMemcpyAsync(ctx->h_status, ctx->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
     CK(ctx, cudaStreamSynchronize(ctx->stream));
-    if (*ctx->h_status & slr::kStatusTimeout)
+    if (reports && (*ctx->h_status & slr::kStatusTimeout))
         return fail(ctx, SLR_ETIMEOUT, "a bounded wait on the tensor core gave up; the bounds are incomplete");
     return SLR_OK;
 }
