@@ -18,12 +18,20 @@
 // absolute weights and the relaxation's arithmetic).  The block form spends its
 // time on scalar shared-memory loads (two per FMA pair) and on barriers between
 // phases of a few boxes.  5-6x50-5 network, block form -> this one: 8,192 boxes
-// with weight gradients 1.65 -> 0.61 ms, 1,000 boxes at supplied slopes 261 -> 113 us,
-// one box 131 -> 94 us, 4,096 boxes' slopes over 20 Adam steps (the sound bounds of
-// every step included) 13.9 -> 5.6 ms; 2-3x32-1, 12,000 boxes 467 -> 217 us.  No
+// with weight gradients 1.65 -> 0.55 ms, 1,000 boxes at supplied slopes 261 -> 101 us,
+// one box 131 -> 87 us, 4,096 boxes' slopes over 20 Adam steps (the sound bounds of
+// every step included) 13.9 -> 4.95 ms; 2-3x32-1, 12,000 boxes 467 -> 216 us.  No
 // shape of its range was slower (one box to 12,000, widths 8 to 128), so the
 // block form serves only networks outside it: more inputs (a row no longer fits
 // a lane's registers), wider layers, or weights beyond shared memory.
+//
+// One block per SM, whose warps share one copy of the weights, and as few of
+// them take boxes as keep the number of rounds: the rounds are full, whatever
+// the number of boxes.  (Three blocks of eight warps per SM, filled one after
+// another, left 4,096 boxes a second round of 448 boxes on a third of the SMs:
+// 196 -> 166 us a pass without that; 100 boxes ran on 13 SMs: 114 -> 93 us, with
+// weight gradients, seven blocks of 16, 250 -> 169 us; 8,192 boxes with weight
+// gradients on 18 warps in three rounds instead of 16 in four 606 -> 550 us.)
 //
 // Weight gradients are sums over boxes: the warps of a CTA meet at each layer
 // and the block adds all its boxes' outer products into accumulators in
@@ -197,8 +205,15 @@ __device__ __forceinline__ void weight_products(const float *X, const float *G, 
     }
 }
 
+// Most threads of a block (one block per SM): as many warps as the registers
+// allow with little spilling (5-6x50-5, 20,000 boxes: 28 warps at 72 registers
+// 590 us, 24 at 80 637 us).
+constexpr int adj_threads(int QP, int RPL, bool w) {
+    return w ? (RPL > 2 || QP == 4 ? 512 : 640) : (RPL > 2 ? 256 : (QP <= 6 ? 896 : 768));
+}
+
 template <int QP, int RPL, bool kW>
-__global__ void __launch_bounds__(kW ? 512 : 256, !kW && QP <= 8 && RPL <= 2 ? 3 : 1)
+__global__ void __launch_bounds__(adj_threads(QP, RPL, kW), 1)
 adj_warp_kernel(const AdjArgs a, const AdjWarpPlan pl, float *chk) {
     extern __shared__ __align__(16) float smem_aw[];
     const NetParams<float> &net = a.net;
@@ -215,7 +230,7 @@ adj_warp_kernel(const AdjArgs a, const AdjWarpPlan pl, float *chk) {
     float *const sm = mine + (kW ? 2 : 1) * pl.rows, *const sr = sm + QP;
     float *const lo = sr + QP, *const hi = lo + R, *const glo = hi + R, *const ghi = glo + R;
     float4 *const ck = reinterpret_cast<float4 *>(chk) +
-                       (size_t)(blockIdx.x * nw + warp) * (K - 1) * RPL * (QP / 2) * 32 + lane;
+                       ((size_t)blockIdx.x * pl.act + warp) * (K - 1) * RPL * (QP / 2) * 32 + lane;
 
     for (int k = 0; k < K; ++k) {
         const int n_in = net.n[k], n_out = net.n[k + 1], ld = pl.w_ld[k];
@@ -237,10 +252,13 @@ adj_warp_kernel(const AdjArgs a, const AdjWarpPlan pl, float *chk) {
         const int64_t c = (int64_t)*a.count;
         n = c < n ? c : n;
     }
-    for (int64_t pos0 = (int64_t)blockIdx.x * nw; pos0 < n; pos0 += (int64_t)gridDim.x * nw) {
-        const int64_t pos = pos0 + warp;
-        const bool live = pos < n;
-        const int nbox = n - pos0 < nw ? (int)(n - pos0) : nw;
+    // kW: neighbouring boxes to a block; else boxes go to the blocks first, then to
+    // their warps, so that few boxes (a.count) and the last round's spread over the SMs
+    const int64_t first = kW ? (int64_t)blockIdx.x * pl.act : blockIdx.x;
+    for (int64_t pos0 = first; pos0 < n; pos0 += (int64_t)gridDim.x * pl.act) {
+        const int64_t pos = kW ? pos0 + warp : pos0 + (int64_t)warp * gridDim.x;
+        const bool live = warp < pl.act && pos < n;
+        const int nbox = n - pos0 < pl.act ? (int)(n - pos0) : pl.act;   // kW: the block's boxes
         if (!kW && !live) continue;
         AdjRows<QP, RPL> rw;
         if (live) {
@@ -658,7 +676,7 @@ void adj_warp_plan(const NetParams<float> &net, int sms, size_t smem_max, AdjWar
     p.rows = widest * 2 * p.QP;
     for (int w = 0; w < 2; ++w) {
         p.box[w] = ((w ? 2 : 1) * p.rows + 2 * p.QP + 4 * net.R + 3) & ~3;
-        for (int nt = w ? 512 : 256; nt >= 64; nt /= 2) {
+        for (int nt = adj_threads(p.QP, p.RPL, w != 0); nt >= 64; nt -= 32) {
             p.threads[w] = nt;
             const size_t smem = smem_of(p, w != 0);
             if (smem > smem_max) continue;
@@ -678,13 +696,18 @@ void adj_warp_plan(const NetParams<float> &net, int sms, size_t smem_max, AdjWar
 cudaError_t launch_adj_warp(const AdjArgs &a, const AdjWarpPlan &p, bool w, float *chk, cudaStream_t s) {
     AdjWarpKernel k = pick(p, w);
     if (k == nullptr || p.grid[w ? 1 : 0] <= 0) return cudaErrorInvalidValue;
-    const int nt = p.threads[w ? 1 : 0], nw = nt / 32;
+    const int nt = p.threads[w ? 1 : 0];
     const size_t smem = smem_of(p, w);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int64_t need = (a.n + nw - 1) / nw;
-    const int grid = (int)(need < p.grid[w ? 1 : 0] ? (need < 1 ? 1 : need) : p.grid[w ? 1 : 0]);
-    k<<<grid, nt, smem, s>>>(a, p, chk);
+    const int64_t most = p.grid[w ? 1 : 0];
+    const int64_t grid = a.n < most ? (a.n < 1 ? 1 : a.n) : most;
+    // the warps that take boxes: as few as keep the rounds, so that the rounds are full
+    AdjWarpPlan pl = p;
+    const int64_t n = a.n < 1 ? 1 : a.n;
+    const int64_t rounds = (n + grid * (nt / 32) - 1) / (grid * (nt / 32));
+    pl.act = (int)((n + grid * rounds - 1) / (grid * rounds));
+    k<<<(int)grid, nt, smem, s>>>(a, pl, chk);
     return cudaGetLastError();
 }
 

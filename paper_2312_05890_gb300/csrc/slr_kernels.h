@@ -115,6 +115,7 @@ struct AdjWarpPlan {
     int rows;                       // floats of one box's rows (widest layer x 2 QP)
     int box[2];                     // floats of one warp's shared memory
     int threads[2], grid[2];        // block size, largest grid (0: the network does not fit)
+    int act;                        // warps of a block that take boxes (set by launch_adj_warp)
     int w_off[kMaxLayers], w_ld[kMaxLayers], b_off[kMaxLayers];
 };
 void adj_warp_plan(const NetParams<float> &net, int sms, size_t smem_max, AdjWarpPlan &p);

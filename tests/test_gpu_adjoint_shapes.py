@@ -79,3 +79,32 @@ def test_adjoint_over_shapes(pkg, d, hidden, out, free):
         for key, got, want in checks:
             ok, e = _close(got, want, 2e-3)
             assert ok, (key, i, e)
+
+
+@pytest.mark.parametrize("per_sm", [0, 1, 16, 20, 28])
+@pytest.mark.parametrize("weights", [False, True])
+def test_adjoint_rounds(pkg, per_sm, weights):
+    """Around a full round of one block per SM: every box is taken once, in whatever slot."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    p = _problem(5, [40, 33], 4, 11)
+    rng = np.random.default_rng(per_sm)
+    with pkg.Counter(0) as c:
+        c.set_problem(p)
+        for n in (per_sm * sms + 1, max(per_sm, 1) * sms, max(per_sm, 1) * sms - 1):
+            lo, hi = random_sub_boxes(p, n, seed=n)
+            g_lo, g_hi = (rng.normal(size=(n, 3)).astype(np.float32) for _ in range(2))
+            a = c.margin_backward(lo, hi, g_lo, g_hi, weights=weights)
+            b = c.margin_backward(lo[::-1], hi[::-1], g_lo[::-1], g_hi[::-1], weights=weights)
+            for key in ("row_lo", "row_hi", "d_lo", "d_hi"):
+                assert np.array_equal(a[key], b[key][::-1]), (key, n)
+            if weights:
+                same = [np.repeat(x[:1], n, axis=0) for x in (lo, hi, g_lo, g_hi)]
+                one = c.margin_backward(*[x[:1] for x in same], weights=True)
+                many = c.margin_backward(*same, weights=True)
+                for key in ("d_W", "d_b"):
+                    for k in range(len(p.net.W)):
+                        want = n * one[key][k].astype(np.float64)
+                        # as above: n equal terms, 2 (d + 1) additions inside each
+                        tol = 2.0 * (n + 2 * 6 + 8) * 2.0 ** -24 * np.abs(want).max() + 1e-30
+                        assert np.abs(many[key][k] - want).max() <= tol, (key, k, n)
