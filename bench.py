@@ -409,7 +409,7 @@ def main():
         tf32_peak = peaks["bf16_tflops"] * TF32_PER_BF16
         ach = gemm_flop / (gemm_ms / 1e3) / 1e12
         roofline = {"bound": "tensor", "achieved": ach, "peak": tf32_peak, "unit": "TFLOP/s",
-                    "frac": ach / tf32_peak, "traffic": None, "kernel": "wide_gemm_kernel (tcgen05 kind::tf32)",
+                    "frac": ach / tf32_peak, "traffic": None, "kernel": "wide_layer_kernel (tcgen05 kind::tf32)",
                     "peak_basis": f"measured bf16 burst {peaks['bf16_tflops']} TFLOP/s x nominal TF32/BF16 "
                                   f"ratio {TF32_PER_BF16:.3f}",
                     "flop_basis": "2 M K (2d + 1) per box and layer (W C on d columns, |W| R on d + 1); "

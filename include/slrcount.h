@@ -100,6 +100,8 @@ typedef struct {
                                (the rest keep fixed slopes); default 1<<16 */
     int32_t tile_boxes;     /* FP32 evaluation kernel: boxes per CTA (64, 32, 16, 8 or 4) and */
     int32_t tile_threads;   /* threads per CTA (256 or 128); 0, 0 = chosen by timing (default).
+                               Levels of few boxes run smaller tiles of 256 threads, so that
+                               their boxes spread over the GPU.
                                A pair the network cannot run with gives SLR_EUNSUPPORTED. */
     int32_t wide;           /* 1: always use the wide path (per-box state in GPU memory, each
                                layer one tensor-core product, no FP64 re-check); 0 (default):

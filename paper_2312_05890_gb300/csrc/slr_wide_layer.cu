@@ -36,8 +36,8 @@
 // Measured on 784-3x256-10, 1,000 boxes (two layers of 1.6 GB read and written):
 // 1.29 ms a layer, tensor pipe 45 % busy, 2.5 TB/s; the rest of a tile's 27 us
 // is the drain (the product waits for its tensor memory, about 5 us) and the
-// producers' loads.  The whole bounds 8.83 -> 3.67 ms, a depth-12 count
-// 76.0 -> 34 ms against one product kernel and one relaxation kernel in place
+// producers' loads.  The whole bounds 8.83 -> 3.66 ms, a depth-12 count
+// 76.0 -> 31.0 ms against one product kernel and one relaxation kernel in place
 // per layer (slr_wide.cu), which still serves fewer than kWideLayerMinD inputs
 // (a column tile of one box would be mostly padding: 70 inputs 1.53 -> 1.17 ms
 // for 3,000 boxes of a 70-2x200-10 network) and more than 16 property rows.
