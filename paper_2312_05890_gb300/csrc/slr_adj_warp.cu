@@ -13,7 +13,7 @@
 // are staged once per CTA, row stride odd, so that both directions read them
 // without bank conflicts.
 //
-// What bounds it: issue slots (54 % active at 24 warps per SM; the packed FMAs
+// What bounds it: issue slots (65 % active at 27 warps per SM; the packed FMAs
 // are a quarter of the instructions, the rest are the loads, the repeated and
 // absolute weights and the relaxation's arithmetic).  The block form spends its
 // time on scalar shared-memory loads (two per FMA pair) and on barriers between
