@@ -415,6 +415,15 @@ int ensure_stage(slr_ctx *ctx, size_t bytes) {
     return SLR_OK;
 }
 
+// Pageable host memory to the device, in the order of the context's stream and
+// with `src` free to go afterwards.  (A copy on the default stream may return
+// before its data has arrived, and the context's stream, which does not wait
+// for the default one, could read the buffer too soon.)
+cudaError_t upload(slr_ctx *ctx, void *dst, const void *src, size_t bytes) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->stream);
+}
+
 float tf32_host(float x) {
     uint32_t u;
     std::memcpy(&u, &x, 4);
@@ -486,7 +495,7 @@ int build_tc(slr_ctx *ctx, const HostLayers<float> &L) {
         ctx->tc_buf = nullptr;
     }
     CK(ctx, cudaMalloc(&ctx->tc_buf, total));
-    CK(ctx, cudaMemcpy(ctx->tc_buf, img.data(), total, cudaMemcpyHostToDevice));
+    CK(ctx, upload(ctx, ctx->tc_buf, img.data(), total));
     ctx->h2d_pending += (int64_t)total;
     for (int k = 1; k < K; ++k) tp.img[k] = (const unsigned char *)ctx->tc_buf + offs[k];
     // the most boxes per CTA whose B operand fits N <= 256 and shared memory
@@ -689,7 +698,7 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
             fill_pieces(L, k, n_in, n_out, Kpad, ctx->wt_Kpad[k], host.data() + offs[k], host.data() + offs_t[k]);
         }
         CK(ctx, cudaMalloc(&ctx->wide_img, total));
-        CK(ctx, cudaMemcpy(ctx->wide_img, host.data(), host_total, cudaMemcpyHostToDevice));
+        CK(ctx, upload(ctx, ctx->wide_img, host.data(), host_total));
         ctx->h2d_pending += (int64_t)host_total;
         ctx->w0t = (const float *)ctx->wide_img;
         ctx->w0b = (const float *)((const unsigned char *)ctx->wide_img + off_w0b);
@@ -2471,9 +2480,12 @@ int slr_leaves(slr_ctx *ctx, int64_t cap, uint64_t *codes, uint8_t *depth, uint8
     const int64_t m = std::min(std::min(cap, ctx->n_leaves), ctx->leaf_cap_alloc);
     CK(ctx, cudaSetDevice(ctx->device));
     if (m > 0) {
-        if (codes) CK(ctx, cudaMemcpy(codes, ctx->leaf_codes, (size_t)m * sizeof(uint64_t), cudaMemcpyDeviceToHost));
-        if (depth) CK(ctx, cudaMemcpy(depth, ctx->leaf_depth, (size_t)m, cudaMemcpyDeviceToHost));
-        if (cls) CK(ctx, cudaMemcpy(cls, ctx->leaf_cls, (size_t)m, cudaMemcpyDeviceToHost));
+        const cudaMemcpyKind back = cudaMemcpyDeviceToHost;
+        if (codes)
+            CK(ctx, cudaMemcpyAsync(codes, ctx->leaf_codes, (size_t)m * sizeof(uint64_t), back, ctx->stream));
+        if (depth) CK(ctx, cudaMemcpyAsync(depth, ctx->leaf_depth, (size_t)m, back, ctx->stream));
+        if (cls) CK(ctx, cudaMemcpyAsync(cls, ctx->leaf_cls, (size_t)m, back, ctx->stream));
+        CK(ctx, cudaStreamSynchronize(ctx->stream));
     }
     if (ctx->n_leaves > ctx->leaf_cap_alloc)
         return fail(ctx, SLR_EOVERFLOW, "%lld leaves exceeded leaf_cap=%lld", (long long)ctx->n_leaves,
@@ -2895,11 +2907,11 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
                 o2.status = bs->status;
             }
         }
-        CK(ctx, cudaMemcpy(A + o_sm, sm.data(), sm.size() * sizeof(slr::BoxSource), cudaMemcpyHostToDevice));
-        CK(ctx, cudaMemcpy(A + o_sr, sr.data(), sr.size() * sizeof(slr::BoxSource), cudaMemcpyHostToDevice));
-        CK(ctx, cudaMemcpy(A + o_om, om.data(), om.size() * sizeof(slr::EvalOutputs), cudaMemcpyHostToDevice));
-        CK(ctx, cudaMemcpy(A + o_or, orr.data(), orr.size() * sizeof(slr::EvalOutputs), cudaMemcpyHostToDevice));
-        CK(ctx, cudaMemcpy(A + o_ca, ca.data(), ca.size() * sizeof(slr::CompactArgs), cudaMemcpyHostToDevice));
+        CK(ctx, upload(ctx, A + o_sm, sm.data(), sm.size() * sizeof(slr::BoxSource)));
+        CK(ctx, upload(ctx, A + o_sr, sr.data(), sr.size() * sizeof(slr::BoxSource)));
+        CK(ctx, upload(ctx, A + o_om, om.data(), om.size() * sizeof(slr::EvalOutputs)));
+        CK(ctx, upload(ctx, A + o_or, orr.data(), orr.size() * sizeof(slr::EvalOutputs)));
+        CK(ctx, upload(ctx, A + o_ca, ca.data(), ca.size() * sizeof(slr::CompactArgs)));
 
         // ---- capture the step loop ----------------------------------------
         int64_t maxcap = 1;
@@ -3457,8 +3469,8 @@ int slr_internal_split_root(slr_ctx *ctx, const slr::BoxSource &root, int64_t *l
     std::sort(set.begin(), set.end());
     std::vector<int8_t> of(d, (int8_t)-1);
     for (int j = 0; j < ns; ++j) of[set[j]] = (int8_t)j;
-    CK(ctx, cudaMemcpy(split_of, of.data(), (size_t)d, cudaMemcpyHostToDevice));
-    CK(ctx, cudaMemcpy(dims_dev, set.data(), (size_t)ns * sizeof(int), cudaMemcpyHostToDevice));
+    CK(ctx, upload(ctx, split_of, of.data(), (size_t)d));
+    CK(ctx, upload(ctx, dims_dev, set.data(), (size_t)ns * sizeof(int)));
     ctx->split_set = set;
     return SLR_OK;
 }
