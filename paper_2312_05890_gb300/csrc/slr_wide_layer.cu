@@ -99,23 +99,32 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 
 // A finite x as TF32 hi + lo, rounded to nearest, ties away from zero (as
 // cvt.rna.tf32.f32, in fewer instructions: half a unit is added to the bits).
-// A NaN does not keep: the bounds do not need it to, since a row that holds
-// one has a NaN or an infinity in its N, which reaches every later row's error
-// bound through the products of the N and E columns (small_row).
+// For the sound bounds only: a NaN may come out as a zero (0x7fffffff, the NaN
+// that FP32 arithmetic gives, carries into the sign).  They do not need it,
+// since a row that holds one has a NaN or an infinity in its N, which reaches
+// every later row's error bound through the products of the N and E columns
+// (small_row).  The adjoint has no such columns and keeps the conversion: a
+// NaN of the caller's or of a state that overflowed is one in what depends on it.
 __device__ __forceinline__ float tf32_bits(float x) {
     return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
 }
 
+template <bool kPlain>
+__device__ __forceinline__ float tf32_piece(float x) {
+    return kPlain ? tf32_rna(x) : tf32_bits(x);
+}
+
+template <bool kPlain>
 __device__ __forceinline__ void split4(const float (&v)[4], unsigned char *hi, unsigned char *lo) {
     float4 h, l;
-    h.x = tf32_bits(v[0]);
-    h.y = tf32_bits(v[1]);
-    h.z = tf32_bits(v[2]);
-    h.w = tf32_bits(v[3]);
-    l.x = tf32_bits(v[0] - h.x);
-    l.y = tf32_bits(v[1] - h.y);
-    l.z = tf32_bits(v[2] - h.z);
-    l.w = tf32_bits(v[3] - h.w);
+    h.x = tf32_piece<kPlain>(v[0]);
+    h.y = tf32_piece<kPlain>(v[1]);
+    h.z = tf32_piece<kPlain>(v[2]);
+    h.w = tf32_piece<kPlain>(v[3]);
+    l.x = tf32_piece<kPlain>(v[0] - h.x);
+    l.y = tf32_piece<kPlain>(v[1] - h.y);
+    l.z = tf32_piece<kPlain>(v[2] - h.z);
+    l.w = tf32_piece<kPlain>(v[3] - h.w);
     *reinterpret_cast<float4 *>(hi) = h;
     *reinterpret_cast<float4 *>(lo) = l;
 }
@@ -342,8 +351,8 @@ __global__ void __launch_bounds__(kLThreads, 1) wide_layer_kernel(const WideLaye
                 }
                 if (cc < NC) {
                     unsigned char *o = to + (cc >> 3) * kLSboB + (cc & 7) * 16;
-                    split4(c, o, o + bimg);
-                    split4(r, o + 2 * bimg, o + 3 * bimg);
+                    split4<kPlain>(c, o, o + bimg);
+                    split4<kPlain>(r, o + 2 * bimg, o + 3 * bimg);
                 }
             }
             if (++st == nst) {
