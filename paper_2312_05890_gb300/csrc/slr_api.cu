@@ -180,6 +180,7 @@ struct slr_ctx {
     std::vector<cudaEvent_t> prof_ev;   // profile: one event before and after each launch
     slr::LevelCounters *h_ctr = nullptr;
     unsigned int *h_status = nullptr;
+    int wait_on_next = 0;                 // polls of the self-check wait in the next wide call (slr_internal_wait_on_next)
     unsigned char *h_stage = nullptr;     // pinned staging for host-to-device copies
     size_t h_stage_bytes = 0;
     int64_t h2d_pending = 0;              // bytes uploaded since the last count returned
@@ -521,6 +522,29 @@ int build_tc(slr_ctx *ctx, const HostLayers<float> &L) {
 
 int ensure_scratch(slr_ctx *ctx, size_t bytes);
 
+// The word that kernels report to (kStatus bits) and its copy on the host.
+int ensure_status(slr_ctx *ctx) {
+    if (!ctx->status) CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
+    if (!ctx->h_status) CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
+    return SLR_OK;
+}
+
+int clear_status(slr_ctx *ctx) {
+    const int rc = ensure_status(ctx);
+    if (rc) return rc;
+    CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned int), ctx->stream));
+    return SLR_OK;
+}
+
+// Waits for the stream; SLR_ETIMEOUT where a bounded wait has given up since clear_status.
+int finish_status(slr_ctx *ctx, const char *what) {
+    CK(ctx, cudaMemcpyAsync(ctx->h_status, ctx->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
+    CK(ctx, cudaStreamSynchronize(ctx->stream));
+    if (*ctx->h_status & slr::kStatusTimeout)
+        return fail(ctx, SLR_ETIMEOUT, "a bounded wait on the tensor core gave up; %s incomplete", what);
+    return SLR_OK;
+}
+
 // Time every tile choice of the FP32 kernel on a fixed set of boxes (sides 1/16
 // of the root box, or of [-0.05, 0.05]^d without one) and keep the fastest.
 // The result is kept per network shape, so new weights of the same shape reuse it.
@@ -572,9 +596,9 @@ int autotune(slr_ctx *ctx, const std::vector<TileChoice> &cands, TileChoice &bes
     src.cap = n;
     slr::EvalOutputs o{};
     o.cls = dcls;
-    if (!ctx->status) {
-        CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
-        CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
+    {
+        const int rc = ensure_status(ctx);
+        if (rc) return rc;
     }
     o.status = ctx->status;
     // each choice on as many boxes as fill whole rounds of its grid (where a
@@ -756,10 +780,19 @@ int ensure_wide_buf(slr_ctx *ctx) {
     return SLR_OK;
 }
 
+// The self-check's wait (on a barrier that nothing completes) among the kernels
+// of the next wide call: how a test sees that a wait that gave up is reported.
+cudaError_t wait_if_asked(slr_ctx *ctx, unsigned int *status) {
+    const int limit = ctx->wait_on_next;
+    ctx->wait_on_next = 0;
+    return limit > 0 ? slr::launch_wait_selfcheck(status, limit, ctx->stream) : cudaSuccess;
+}
+
 // Bound positions [0, n) of `src` on the wide path, chunk by chunk.
 int run_wide(slr_ctx *ctx, const slr::BoxSource &src, int64_t n, const slr::EvalOutputs &out, int64_t *launches) {
     int rc = ensure_wide_buf(ctx);
     if (rc) return rc;
+    CK(ctx, wait_if_asked(ctx, out.status));
     const slr::NetParams<float> &nf = ctx->nf;
     const int K = nf.K, d = nf.d, np = ctx->wide_NP, R = nf.R, sms = ctx->sm_count;
     const size_t bc = (size_t)ctx->wide_Bc;
@@ -920,10 +953,7 @@ int run_wide_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int64_t *launches) {
         n = std::min<int64_t>(n, (int64_t)c);
     }
     if (n <= 0) return SLR_OK;
-    if (!ctx->status) {
-        CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
-        CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
-    }
+    CK(ctx, wait_if_asked(ctx, ctx->status));
     // chunk: the boxes whose state fits about 6 GB
     const size_t eq = (size_t)Q * np;
     const size_t per_box = sizeof(float) * (eq * (size_t)(2 * (K - 1) - 1 + 6) + 5 * (size_t)(K - 1) * np +
@@ -1339,10 +1369,10 @@ int ensure_count_buffers(slr_ctx *ctx) {
     }
     if (!ctx->ctr) {
         CK(ctx, cudaMalloc(&ctx->ctr, sizeof(slr::LevelCounters)));
-        CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
         CK(ctx, cudaMallocHost(&ctx->h_ctr, sizeof(slr::LevelCounters)));
-        CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
     }
+    const int rc = ensure_status(ctx);
+    if (rc) return rc;
     const int d = ctx->widths[0];
     if (ctx->root_d != d) {
         cudaFree(ctx->root);
@@ -2434,16 +2464,13 @@ int slr_bounds(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi
     o.row_lo = drl;
     o.row_hi = drh;
     o.row_err = dre;
-    if (!ctx->status) {
-        CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
-        CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
-    }
+    if ((rc = ensure_status(ctx))) return rc;
     o.status = ctx->status;
     // only the tensor-core paths report through the status word here (the FP32
     // tile writes it when a re-check list overflows, and bounds have none)
     const bool tc = ctx->opt.precision == SLR_PREC_TC_TF32 && ctx->tc_ok && alpha == nullptr;
     const bool reports = ctx->wide || tc;
-    if (reports) CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned int), ctx->stream));
+    if (reports && (rc = clear_status(ctx))) return rc;
     if (ctx->wide) {
         int64_t launches = 0;
         if ((rc = run_wide(ctx, src, n, o, &launches))) return rc;
@@ -2465,11 +2492,8 @@ int slr_bounds(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi
             CK(ctx, cudaMemcpyAsync(row_err, dre, (size_t)n * R * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
         if (cls) CK(ctx, cudaMemcpyAsync(cls, dcls, (size_t)n, cudaMemcpyDeviceToHost, ctx->stream));
     }
-    if (reports)
-        CK(ctx, cudaMemcpyAsync(ctx->h_status, ctx->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
+    if (reports) return finish_status(ctx, "the bounds are");
     CK(ctx, cudaStreamSynchronize(ctx->stream));
-    if (reports && (*ctx->h_status & slr::kStatusTimeout))
-        return fail(ctx, SLR_ETIMEOUT, "a bounded wait on the tensor core gave up; the bounds are incomplete");
     return SLR_OK;
 }
 
@@ -2518,6 +2542,13 @@ int slr_wait_selfcheck(slr_ctx *ctx, int32_t limit) {
     if (e != cudaSuccess) return fail(ctx, SLR_ECUDA, "%s", cudaGetErrorString(e));
     if (st & slr::kStatusTimeout)
         return fail(ctx, SLR_ETIMEOUT, "a bounded device wait gave up after %d polls", limit);
+    return SLR_OK;
+}
+
+int slr_internal_wait_on_next(slr_ctx *ctx, int32_t limit) {
+    if (!ctx) return fail(nullptr, SLR_EINVAL, "null context");
+    if (limit < 1 || limit > (1 << 20)) return fail(ctx, SLR_EINVAL, "limit %d out of range [1, 2^20]", limit);
+    ctx->wait_on_next = limit;
     return SLR_OK;
 }
 
@@ -3611,6 +3642,9 @@ int slr_margin_backward(slr_ctx *ctx, int64_t n, const float *box_lo, const floa
             CK(ctx, cudaMemsetAsync(db[k], 0, (size_t)ctx->widths[k + 1] * sizeof(float), ctx->stream));
         }
     }
+    // (the wide path's products have bounded waits; with weight gradients one block takes a box)
+    const bool reports = n > 0 && ctx->wide && !want_w;
+    if (reports && (rc = clear_status(ctx))) return rc;
     if (n > 0) {
         slr::AdjArgs a = adj_base(ctx);
         a.src.mode = 1;
@@ -3654,6 +3688,7 @@ int slr_margin_backward(slr_ctx *ctx, int64_t n, const float *box_lo, const floa
             }
         }
     }
+    if (reports) return finish_status(ctx, "the gradients are");
     CK(ctx, cudaStreamSynchronize(ctx->stream));
     return SLR_OK;
 }
@@ -3678,11 +3713,7 @@ int slr_optimize_alpha(slr_ctx *ctx, int64_t n, const float *box_lo, const float
     const size_t need = alpha_bytes(n, H, R) + align_up((size_t)n) + (on_device ? 0 : 2 * s_box);
     if (!on_device && (rc = check_boxes(ctx, n, d, box_lo, box_hi))) return rc;
     if ((rc = ensure_scratch(ctx, need))) return rc;
-    if (!ctx->status) {
-        CK(ctx, cudaMalloc(&ctx->status, sizeof(unsigned int)));
-        CK(ctx, cudaMallocHost(&ctx->h_status, sizeof(unsigned int)));
-    }
-    CK(ctx, cudaMemsetAsync(ctx->status, 0, sizeof(unsigned int), ctx->stream));
+    if ((rc = clear_status(ctx))) return rc;
     unsigned char *p = (unsigned char *)ctx->scratch;
     const AlphaBuffers b = carve_alpha(p, n, H, R);
     p += alpha_bytes(n, H, R);
@@ -3713,9 +3744,7 @@ int slr_optimize_alpha(slr_ctx *ctx, int64_t n, const float *box_lo, const float
     }
     if (cls) CK(ctx, cudaMemcpyAsync(cls, dcls, (size_t)n, kind, ctx->stream));
     if (alpha) CK(ctx, cudaMemcpyAsync(alpha, b.alpha, (size_t)n * H * sizeof(float), kind, ctx->stream));
-    CK(ctx, cudaMemcpyAsync(ctx->h_status, ctx->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->stream));
-    CK(ctx, cudaStreamSynchronize(ctx->stream));
-    return SLR_OK;
+    return finish_status(ctx, "the slopes and bounds are");
 }
 
 }  // extern "C"
