@@ -781,25 +781,26 @@ cudaError_t launch_wide_classify(const NetParams<float> &net, int nb, int64_t ba
     return cudaGetLastError();
 }
 
+template <int RM>
+static cudaError_t launch_rows_product(const float *Wt, int n_in, int R, const float *B, int ldb, float *D, int ldd,
+                                       int64_t ncols, bool abs_w, int sms, cudaStream_t s) {
+    // 13 or more rows of more than 768 inputs pass the 48 KB that a launch may use
+    // unasked (the limit asked for is the widest layer's, whatever this call needs)
+    cudaError_t e = cudaFuncSetAttribute(wide_rows_product_kernel<RM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         kMaxWidth * RM * (int)sizeof(float));
+    if (e != cudaSuccess) return e;
+    wide_rows_product_kernel<RM><<<grid_for(ncols, sms), 256, (size_t)n_in * RM * sizeof(float), s>>>(
+        Wt, n_in, R, B, ldb, D, ldd, ncols, abs_w ? 1 : 0);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_wide_rows_product(const float *Wt, int n_in, int R, const float *B, int ldb, float *D, int ldd,
                                      int64_t ncols, bool abs_w, int sms, cudaStream_t s) {
-    const int grid = grid_for(ncols, sms);
-    if (R <= 4) {
-        wide_rows_product_kernel<4><<<grid, 256, (size_t)n_in * 4 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D, ldd,
-                                                                                       ncols, abs_w ? 1 : 0);
-    } else if (R <= 8) {
-        wide_rows_product_kernel<8><<<grid, 256, (size_t)n_in * 8 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D, ldd,
-                                                                                       ncols, abs_w ? 1 : 0);
-    } else if (R <= 12) {
-        wide_rows_product_kernel<12><<<grid, 256, (size_t)n_in * 12 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D,
-                                                                                         ldd, ncols, abs_w ? 1 : 0);
-    } else if (R <= 16) {
-        wide_rows_product_kernel<16><<<grid, 256, (size_t)n_in * 16 * sizeof(float), s>>>(Wt, n_in, R, B, ldb, D,
-                                                                                         ldd, ncols, abs_w ? 1 : 0);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    if (R <= 4) return launch_rows_product<4>(Wt, n_in, R, B, ldb, D, ldd, ncols, abs_w, sms, s);
+    if (R <= 8) return launch_rows_product<8>(Wt, n_in, R, B, ldb, D, ldd, ncols, abs_w, sms, s);
+    if (R <= 12) return launch_rows_product<12>(Wt, n_in, R, B, ldb, D, ldd, ncols, abs_w, sms, s);
+    if (R <= 16) return launch_rows_product<16>(Wt, n_in, R, B, ldb, D, ldd, ncols, abs_w, sms, s);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_wait_selfcheck(unsigned int *status, int limit, cudaStream_t s) {
