@@ -682,7 +682,7 @@ void adj_warp_plan(const NetParams<float> &net, int sms, size_t smem_max, AdjWar
             if (smem > smem_max) continue;
             AdjWarpKernel k = pick(p, w != 0);
             int nb = 0;
-            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            if (allow_smem(k) != cudaSuccess ||
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, nt, smem) != cudaSuccess) {
                 (void)cudaGetLastError();
                 nb = 0;
@@ -698,7 +698,7 @@ cudaError_t launch_adj_warp(const AdjArgs &a, const AdjWarpPlan &p, bool w, floa
     if (k == nullptr || p.grid[w ? 1 : 0] <= 0) return cudaErrorInvalidValue;
     const int nt = p.threads[w ? 1 : 0];
     const size_t smem = smem_of(p, w);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     const int64_t most = p.grid[w ? 1 : 0];
     const int64_t grid = a.n < most ? (a.n < 1 ? 1 : a.n) : most;

@@ -807,8 +807,7 @@ cudaError_t launch_adjoint(const AdjArgs &a, int grid, cudaStream_t s) {
         return cudaGetLastError();
     }
     const size_t smem = adjoint_smem_bytes(a);
-    cudaError_t e = cudaFuncSetAttribute(slr_adjoint_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = allow_smem(slr_adjoint_kernel<false>);
     if (e != cudaSuccess) return e;
     slr_adjoint_kernel<false><<<grid, 256, smem, s>>>(a);
     return cudaGetLastError();
@@ -816,8 +815,8 @@ cudaError_t launch_adjoint(const AdjArgs &a, int grid, cudaStream_t s) {
 
 int adjoint_blocks_per_sm(size_t smem) {
     int nb = 0;
-    cudaFuncSetAttribute(slr_adjoint_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, slr_adjoint_kernel<false>, 256, smem) != cudaSuccess)
+    if (allow_smem(slr_adjoint_kernel<false>) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, slr_adjoint_kernel<false>, 256, smem) != cudaSuccess)
         return 0;
     return nb;
 }

@@ -20,7 +20,7 @@ namespace {
 thread_local std::string g_create_error;
 
 constexpr size_t kAlign = 256;
-constexpr int kMaxSmem = 232448;   // 227 KB of dynamic shared memory per CTA
+constexpr int kMaxSmem = slr::kCtaSmem;
 
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
@@ -2662,11 +2662,10 @@ TileShape problem_shape(const ProblemHost &h) {
 // 32, 16, 8, 4 whose product tiles fit two per thread and whose shared memory
 // fits next to a problem's shared copies.
 constexpr int kBatchTiles[] = {32, 16, 8, 4};
-constexpr size_t kBatchStatic = 4096;
 int batch_tile_for(const TileShape &s) {
     for (int t : kBatchTiles)
         if (slr::eval_gemm_items(t, s.d, s.nmp) <= 2 * 256 &&
-            slr::eval_smem_bytes<float>(t, s.d, s.R, s.nmp, s.n_in) + kBatchStatic <= (size_t)kMaxSmem)
+            slr::eval_smem_bytes<float>(t, s.d, s.R, s.nmp, s.n_in) + slr::kBatchStatic <= (size_t)kMaxSmem)
             return t;
     return 0;
 }
@@ -2816,14 +2815,13 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
         std::memcpy(bs->h_upload + o_n64, n64.data(), (size_t)P * sizeof(slr::NetParams<double>));
 
         // ---- tiles: the most boxes in flight that the largest problem allows ----
-        const size_t kStatic = 4096;   // shared copies of one problem's params, source and outputs
         auto pick = [&](bool f64, int &T, size_t &smem, int &grid) {
             T = 0;
             long best = 0;
             for (int t : slr::kTileSizes) {
                 const size_t sm = f64 ? slr::eval_smem_bytes<double>(t, sh64.d, sh64.R, sh64.nmp, sh64.n_in_max)
                                       : slr::eval_smem_bytes<float>(t, sh32.d, sh32.R, sh32.nmp, sh32.n_in_max);
-                if (sm + kStatic > (size_t)kMaxSmem) continue;
+                if (sm + slr::kBatchStatic > (size_t)kMaxSmem) continue;
                 bool fits = true;   // each problem's contraction tiles must fit two per thread
                 for (int i = 0; i < P && fits; ++i)
                     fits = slr::eval_gemm_items(t, n32[i].d, n32[i].n_max_pad) <= 2 * 256;
@@ -2869,7 +2867,7 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
             for (int tt : kBatchTiles) {
                 if (tt > t) continue;
                 const size_t sm = slr::eval_smem_bytes<float>(tt, sh.d, sh.R, sh.nmp, sh.n_in_max);
-                if (sm + kStatic > (size_t)kMaxSmem) continue;
+                if (sm + slr::kBatchStatic > (size_t)kMaxSmem) continue;
                 const int nb = slr::eval_batch_blocks_per_sm_f32(tt, sm);
                 if (nb <= 0) continue;
                 gr.T = tt;
@@ -3149,7 +3147,7 @@ static bool batch_tile_fits(const slr_problem &q) {
     }
     const int nmp = (nmax + 7) & ~7;
     return slr::eval_gemm_items(4, d, nmp) <= 2 * 256 &&
-           slr::eval_smem_bytes<float>(4, d, R, nmp, nin) + kBatchStatic <= (size_t)kMaxSmem;
+           slr::eval_smem_bytes<float>(4, d, R, nmp, nin) + slr::kBatchStatic <= (size_t)kMaxSmem;
 }
 
 extern "C" int slr_count_batch(slr_ctx *ctx, int n, const slr_problem *problems, slr_result *results) {

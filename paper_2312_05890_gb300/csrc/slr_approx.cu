@@ -100,7 +100,7 @@ cudaError_t launch_approx_sample(const NetParams<double> &net, const double *lo,
                                  unsigned long long seed, int trial, int split, int n, double *coord,
                                  unsigned long long *count, int sms, cudaStream_t s) {
     const size_t smem = approx_sample_smem(net);
-    cudaError_t e = cudaFuncSetAttribute(approx_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(approx_sample_kernel);
     if (e != cudaSuccess) return e;
     const int need = (n + kSampleWarps - 1) / kSampleWarps;
     const int grid = need < 4 * sms ? need : 4 * sms;

@@ -8,7 +8,7 @@ template <int T, int NT, int KI, int DC = 0>
 static cudaError_t launch_t(int grid, size_t smem, cudaStream_t s, const NetParams<float> &net,
                             const BoxSource &src, const EvalOutputs &out, int pass) {
     auto k = slr_eval_kernel<float, T, NT, KI, DC>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     k<<<grid, NT, smem, s>>>(net, src, out, pass);
     return cudaGetLastError();
@@ -17,7 +17,7 @@ static cudaError_t launch_t(int grid, size_t smem, cudaStream_t s, const NetPara
 template <int T, int NT, int KI>
 static int occ_t(size_t smem) {
     auto k = slr_eval_kernel<float, T, NT, KI>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (allow_smem(k) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, smem) != cudaSuccess) return 0;
     return nb;
@@ -97,7 +97,7 @@ static cudaError_t launch_batch_t(int grid, size_t smem, cudaStream_t s, const N
                                   const BoxSource *srcs, const EvalOutputs *outs, int P, const long long *prefix,
                                   const BatchShape &shape, int pass) {
     auto k = slr_eval_batch_kernel<float, T, 256>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, kBatchStatic);
     if (e != cudaSuccess) return e;
     k<<<grid, 256, smem, s>>>(nets, srcs, outs, P, prefix, shape, pass);
     return cudaGetLastError();
@@ -106,7 +106,7 @@ static cudaError_t launch_batch_t(int grid, size_t smem, cudaStream_t s, const N
 template <int T>
 static int occ_batch_t(size_t smem) {
     auto k = slr_eval_batch_kernel<float, T, 256>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (allow_smem(k, kBatchStatic) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, 256, smem) != cudaSuccess) return 0;
     return nb;

@@ -8,7 +8,7 @@ template <int T, int NT>
 static cudaError_t launch_t(int grid, size_t smem, cudaStream_t s, const NetParams<double> &net,
                             const BoxSource &src, const EvalOutputs &out, int pass) {
     auto k = slr_eval_kernel<double, T, NT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     k<<<grid, NT, smem, s>>>(net, src, out, pass);
     return cudaGetLastError();
@@ -17,7 +17,7 @@ static cudaError_t launch_t(int grid, size_t smem, cudaStream_t s, const NetPara
 template <int T, int NT>
 static int occ_t(size_t smem) {
     auto k = slr_eval_kernel<double, T, NT>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (allow_smem(k) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, NT, smem) != cudaSuccess) return 0;
     return nb;
@@ -73,7 +73,7 @@ template <int T>
 static cudaError_t launch_cluster_t(int grid, size_t smem, cudaStream_t s, const NetParams<double> &net,
                                     const BoxSource &src, const EvalOutputs &out, int pass) {
     auto k = slr_eval_cluster_kernel<double, T, 256>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     k<<<grid, 256, smem, s>>>(net, src, out, pass);
     return cudaGetLastError();
@@ -82,7 +82,7 @@ static cudaError_t launch_cluster_t(int grid, size_t smem, cudaStream_t s, const
 template <int T>
 static int cluster_max_t(size_t smem) {
     auto k = slr_eval_cluster_kernel<double, T, 256>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (allow_smem(k) != cudaSuccess) {
         (void)cudaGetLastError();
         return 0;
     }
@@ -118,7 +118,7 @@ static cudaError_t launch_batch_t(int grid, size_t smem, cudaStream_t s, const N
                                   const BoxSource *srcs, const EvalOutputs *outs, int P, const long long *prefix,
                                   const BatchShape &shape, int pass) {
     auto k = slr_eval_batch_kernel<double, T, 256>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, kBatchStatic);
     if (e != cudaSuccess) return e;
     k<<<grid, 256, smem, s>>>(nets, srcs, outs, P, prefix, shape, pass);
     return cudaGetLastError();
@@ -127,7 +127,7 @@ static cudaError_t launch_batch_t(int grid, size_t smem, cudaStream_t s, const N
 template <int T>
 static int occ_batch_t(size_t smem) {
     auto k = slr_eval_batch_kernel<double, T, 256>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
+    if (allow_smem(k, kBatchStatic) != cudaSuccess) return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, 256, smem) != cudaSuccess) return 0;
     return nb;

@@ -342,7 +342,7 @@ template <int T>
 static cudaError_t launch_tc_t(int grid, size_t smem, cudaStream_t s, const NetParams<float> &net, const TcParams &tc,
                                const BoxSource &src, const EvalOutputs &out, int pass) {
     auto k = slr_eval_tc_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k);
     if (e != cudaSuccess) return e;
     k<<<grid, kTcThreads, smem, s>>>(net, tc, src, out, pass);
     return cudaGetLastError();

@@ -14,6 +14,18 @@ constexpr int kTileSizes[] = {64, 32, 20, 16, 12, 8, 4};
 constexpr int kTcTileSizes[] = {64, 32, 16, 8, 4};
 constexpr int kThreadCounts[] = {256, 128};
 
+constexpr int kCtaSmem = 232448;      // 227 KB: the most shared memory of a CTA
+constexpr int kBatchStatic = 4096;    // of which the batched kernels hold their copies of a problem's parameters
+
+// Lets launches of `kernel`, which holds `fixed` bytes of static shared memory,
+// use the rest of a CTA's.  The limit is the kernel's, for the whole process:
+// set to one launch's need it would fail the launches of other threads, whose
+// contexts run the same kernel for other networks.
+template <class K>
+cudaError_t allow_smem(K *kernel, int fixed = 0) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCtaSmem - fixed);
+}
+
 // Fused evaluation (kernel (b) plus its contraction); one instantiation per
 // working precision.  `T` must be one of kTileSizes and `NT` of kThreadCounts
 // (tiles of 20 and 12 boxes exist in FP32 only).

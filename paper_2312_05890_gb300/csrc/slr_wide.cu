@@ -784,10 +784,8 @@ cudaError_t launch_wide_classify(const NetParams<float> &net, int nb, int64_t ba
 template <int RM>
 static cudaError_t launch_rows_product(const float *Wt, int n_in, int R, const float *B, int ldb, float *D, int ldd,
                                        int64_t ncols, bool abs_w, int sms, cudaStream_t s) {
-    // 13 or more rows of more than 768 inputs pass the 48 KB that a launch may use
-    // unasked (the limit asked for is the widest layer's, whatever this call needs)
-    cudaError_t e = cudaFuncSetAttribute(wide_rows_product_kernel<RM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kMaxWidth * RM * (int)sizeof(float));
+    // (13 or more rows of more than 768 inputs pass the 48 KB that a launch may use unasked)
+    cudaError_t e = allow_smem(wide_rows_product_kernel<RM>);
     if (e != cudaSuccess) return e;
     wide_rows_product_kernel<RM><<<grid_for(ncols, sms), 256, (size_t)n_in * RM * sizeof(float), s>>>(
         Wt, n_in, R, B, ldb, D, ldd, ncols, abs_w ? 1 : 0);
@@ -815,7 +813,7 @@ cudaError_t launch_wide_gemm(const WideGemmArgs &args, int nprob, cudaStream_t s
         gy = std::max(gy, (args.g[i].M + kWM - 1) / kWM);
     }
     const size_t smem = wide_gemm_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(wide_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(wide_gemm_kernel);
     if (e != cudaSuccess) return e;
     wide_gemm_kernel<<<dim3(gx * gy, 1, nprob), kWThreads, smem, s>>>(args, gy);
     return cudaGetLastError();

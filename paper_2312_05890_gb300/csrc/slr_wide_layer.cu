@@ -75,7 +75,6 @@ constexpr int kLThreads = 32 * (kLWork + 2);
 constexpr int kLCols = 2 * 8 * kLWork;            // most columns of a tile: two groups of eight per producer warp
 constexpr int kLTmemR = 256;                      // tensor memory column of R'
 constexpr int kLBar = 256;                        // bytes of the barriers
-constexpr int kLSmemMax = 232448;                 // 227 KB of dynamic shared memory per CTA
 constexpr int kLWait = 1 << 24;
 
 // Bytes of one piece of one equation's operand of a step, and of a whole step
@@ -84,7 +83,7 @@ constexpr int kLWait = 1 << 24;
 __host__ __device__ inline int b_img(int NC) { return NC / 8 * kLSboB; }
 __host__ __device__ inline int b_step(int NC) { return 4 * b_img(NC) + 64; }
 __host__ __device__ inline int b_stage(int NC) { return kLK / kLStep * b_step(NC); }
-inline int a_stages(int NC) { return std::min(kAMax, (kLSmemMax - kLBar - kBStages * b_stage(NC)) / kLA); }
+inline int a_stages(int NC) { return std::min(kAMax, (kCtaSmem - kLBar - kBStages * b_stage(NC)) / kLA); }
 
 // What a producer thread holds between its loads and its stores: four
 // neighbouring inputs of two columns.
@@ -904,7 +903,7 @@ static cudaError_t launch_layer(WideLayer G, int sms, cudaStream_t s) {
     if (items > INT32_MAX) return cudaErrorInvalidValue;
     G.na = a_stages(G.NC);
     const int smem = G.na * kLA + kBStages * b_stage(G.NC) + kLBar;
-    cudaError_t e = cudaFuncSetAttribute(wide_layer_kernel<kPlain>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(wide_layer_kernel<kPlain>);
     if (e != cudaSuccess) return e;
     wide_layer_kernel<kPlain><<<(int)std::min<int64_t>(items, sms), kLThreads, smem, s>>>(G);
     return cudaGetLastError();
@@ -917,9 +916,8 @@ cudaError_t launch_wide_product(const WideLayer &G, int sms, cudaStream_t s) { r
 cudaError_t launch_wide_plan1(const NetParams<float> &net, const float *W0t, int nb, int NP, const float *mh,
                               const float *ml, const float *rr, float *plan, float *S3, float *Ch, float *Cl,
                               const float *alpha, int64_t alpha_ld, int64_t base, cudaStream_t s) {
+    // (12 KB at most: no need to ask for it)
     const int smem = 3 * plan1_run(net.d) * kP1Y * (int)sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(wide_plan1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
     wide_plan1_kernel<<<dim3(NP / kP1X, nb), dim3(kP1X, kP1Y), smem, s>>>(net, W0t, NP, mh, ml, rr, plan, S3, Ch, Cl,
                                                                           alpha, alpha_ld, base);
     return cudaGetLastError();
@@ -948,7 +946,7 @@ cudaError_t launch_wide_rows(const NetParams<float> &net, int nb, int NP, const 
     const int RM = wide_rows_stride(net.R);
     const size_t smem = (size_t)((net.n[net.K - 1] + 31) & ~31) * RM * sizeof(float);
     auto run = [&](auto k) -> cudaError_t {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = allow_smem(k);
         if (e != cudaSuccess) return e;
         k<<<grid, 256, smem, s>>>(net, NP, ntile, NC, Cin, Rin, W0b, rr, plan, ncols, out);
         return cudaGetLastError();
