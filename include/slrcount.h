@@ -98,10 +98,13 @@ typedef struct {
     float alpha_lr;         /* Adam step size of those steps; default 0.1 */
     int64_t alpha_cap;      /* most UNDECIDED boxes per level whose slopes are optimised
                                (the rest keep fixed slopes); default 1<<16 */
-    int32_t tile_boxes;     /* FP32 evaluation kernel: boxes per CTA (64, 32, 16, 8 or 4) and */
-    int32_t tile_threads;   /* threads per CTA (256 or 128); 0, 0 = chosen by timing (default).
-                               Levels of few boxes run smaller tiles of 256 threads, so that
-                               their boxes spread over the GPU.
+    int32_t tile_boxes;     /* FP32 evaluation kernel: boxes per CTA (64, 32, 20, 16, 12, 8 or 4) and */
+    int32_t tile_threads;   /* threads per CTA (256 or 128); 0, 0 = chosen by timing (default):
+                               a count's levels of few boxes then run smaller tiles of 256
+                               threads, so that their boxes spread over the GPU.  A pair set here
+                               runs every level and every call, of few boxes too.  A tile decides
+                               the last bits of a bound (the order of its sums, and the box of the
+                               tile that its constants are taken relative to).
                                A pair the network cannot run with gives SLR_EUNSUPPORTED. */
     int32_t wide;           /* 1: always use the wide path (per-box state in GPU memory, each
                                layer one tensor-core product, no FP64 re-check); 0 (default):
@@ -158,7 +161,8 @@ typedef struct {
     int64_t launches;       /* kernels launched by the count */
     int64_t h2d_bytes;      /* host-to-device bytes copied by the count (inputs, schedule) */
     int64_t d2h_bytes;      /* device-to-host bytes copied by the count (counters, status) */
-    int32_t tile_boxes;     /* boxes per CTA of the FP32 evaluation kernel (chosen by timing) */
+    int32_t tile_boxes;     /* boxes per CTA of the FP32 evaluation kernel (set, or chosen by timing:
+                               then levels of few boxes ran smaller tiles) */
     int32_t tile_threads;   /* threads per CTA of the FP32 evaluation kernel */
     uint64_t rechecked_fp32; /* TC_TF32: boxes re-bounded by the FP32 path */
     uint64_t alpha_boxes;   /* alpha_steps > 0: boxes whose slopes were optimised */
@@ -351,7 +355,7 @@ typedef struct {
  * and stream of its own).  results[i] receives problem i's count as
  * slr_count would return it (device_ms is the time of the whole batch,
  * completion_ms the time from its start to the end of problem i's last level;
- * tile_boxes the problem's tile).
+ * tile_boxes the problem's tile, which runs all its levels).
  * Inputs are copied.  Each problem's frontier holds up to min(2^depth,
  * frontier_cap) boxes (SLR_EOVERFLOW beyond).  Uses the context's options
  * (relax_mode, fp64_recheck, frontier_cap) and stream; FP32 arithmetic with
@@ -411,9 +415,10 @@ int slr_count_noalloc(slr_ctx *ctx, int D, slr_result *out);
  * property and result options (precision, relax_mode, fp64_recheck,
  * recheck_cluster, recheck_pairs, wide), else SLR_EINVAL; a blob that is truncated or not a
  * checkpoint gives SLR_EINVAL.  The blob also records the FP32 tile (boxes
- * and threads per CTA) of the checkpointed levels: the resumed levels run
- * that tile, whatever the context's own choice, because the tile fixes the
- * order of the FP32 sums and so which boxes take the FP64 re-check.  Neither call supports record_leaves, alpha_steps > 0, the
+ * and threads per CTA) of the checkpointed levels, and whether it was set or
+ * chosen by timing: the resumed levels run the tiles of that count, whatever
+ * the context's own choice, because the tile fixes the order of the FP32 sums
+ * and so which boxes take the FP64 re-check.  Neither call supports record_leaves, alpha_steps > 0, the
  * gradient split rule or sharding (SLR_EUNSUPPORTED). */
 int slr_count_checkpoint(slr_ctx *ctx, int D, int t, void *buf, size_t cap, size_t *used);
 int slr_count_resume(slr_ctx *ctx, const void *buf, size_t bytes, slr_result *out);

@@ -4,6 +4,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -98,7 +99,8 @@ struct slr_ctx {
     bool pairs_fit = false;   // the FP64 tile's footprint holds the float-float stage's planes
     size_t smem32 = 0, smem64 = 0;
     int grid32 = 0, grid64 = 0;
-    std::vector<TileChoice> small32;      // the FP32 tiles of 256 threads, ascending (few_tile)
+    std::vector<TileChoice> small32;      // the FP32 tiles of 256 threads, ascending (level_tile)
+    bool small_levels = true;             // levels of few boxes may run them: the caller has set no tile
     int grid64c = 0;   // > 0: the FP64 re-check on clusters (grid of that many CTAs)
     void *tc_buf = nullptr;               // tensor-core weight images
     slr::TcParams tcp{};
@@ -1118,21 +1120,30 @@ std::vector<TileChoice> recheck_candidates(slr_ctx *ctx, bool pairs) {
     return c64;
 }
 
-// The FP32 tile for at most `most` boxes: the smallest tile that still gives
-// every tile an SM of its own, else the context's.  A tile's time grows with
-// its boxes, so few boxes are done soonest on many small tiles: levels 0 to 8
-// of a 5-6x50-5 tanh count take 45 us each on 4-box tiles, 78 us on its 20-box
-// one, the whole depth-16 count 3.66 -> 3.22 ms.  The rule
-// takes nothing but the boxes and the context's tile: a level of a count (at
-// most 2^t boxes) runs the same tile in every form of the count.
-TileChoice few_tile(const slr_ctx *ctx, int64_t most) {
-    for (const TileChoice &c : ctx->small32) {
-        if (c.T >= ctx->T32) break;
-        if ((most + c.T - 1) / c.T <= ctx->sm_count) return c;
-    }
+// SMs of a GB300: a constant, so that a count resumed on a part of one runs the same tiles.
+constexpr int kFewTiles = 152;
+
+// The FP32 tile of level t of a count (at most 2^t boxes).  Where the caller
+// has set a tile, that one.  Else, at levels of few boxes, the smallest tile
+// that still gives every tile an SM of its own: a tile's time grows with its
+// boxes, so few boxes are done soonest on many small tiles (levels 0 to 8 of a
+// 5-6x50-5 tanh count take 45 us each on 4-box tiles, 78 us on its 20-box one,
+// the whole depth-16 count 3.66 -> 3.22 ms).  A tile decides the last bits of a
+// bound, so the rule takes nothing but the level and the context's tile: a
+// level runs the same tile in every form of the count, and bounds and slope
+// steps, which report no tile, run the context's.
+TileChoice context_tile(const slr_ctx *ctx) {
     return TileChoice{ctx->T32, ctx->NT32, ctx->grid32 / std::max(1, ctx->sm_count), ctx->smem32};
 }
-TileChoice level_tile(const slr_ctx *ctx, int t) { return few_tile(ctx, (int64_t)1 << std::min(t, 40)); }
+TileChoice level_tile(const slr_ctx *ctx, int t) {
+    const int64_t most = (int64_t)1 << std::min(t, 40);
+    if (ctx->small_levels)
+        for (const TileChoice &c : ctx->small32) {
+            if (c.T >= ctx->T32) break;
+            if ((most + c.T - 1) / c.T <= kFewTiles) return c;
+        }
+    return context_tile(ctx);
+}
 
 void choose_recheck_tile(slr_ctx *ctx) {
     std::vector<TileChoice> c64 = recheck_candidates(ctx, true);
@@ -1287,6 +1298,7 @@ int prepare_device(slr_ctx *ctx) {
     ctx->NT32 = best.NT;
     ctx->smem32 = best.smem;
     ctx->grid32 = best.blocks * ctx->sm_count;
+    ctx->small_levels = ctx->opt.tile_boxes == 0;
     ctx->small32.clear();
     for (auto c = c32.rbegin(); c != c32.rend(); ++c)
         if (c->NT == 256) ctx->small32.push_back(*c);
@@ -1966,7 +1978,7 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
         if (use_tc) hp = fnv1a(hp, &ctx->tcp, sizeof ctx->tcp);
         char key[640];
         std::snprintf(key, sizeof key,
-                      "%d|%d|%d|%d|%d|%d|%d|%d|%llu|%p|%p|%p|%p|%p|%p|%p|%p|%p|%lld|%lld|%lld|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d",
+                      "%d|%d|%d|%d|%d|%d|%d|%d|%llu|%p|%p|%p|%p|%p|%p|%p|%p|%p|%lld|%lld|%lld|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d|%d",
                       D, leaves ? 1 : 0, recheck ? 1 : 0, use_tc ? 1 : 0, prof ? 1 : 0, ctx->opt.shard_count,
                       ctx->opt.shard_index, shard_g,
                       (unsigned long long)hp, (void *)ctx->codes[0], (void *)ctx->codes[1],
@@ -1974,7 +1986,8 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
                       (void *)ctx->leaf_codes, (void *)ctx->masks, (void *)ctx->root, (long long)ctx->cap,
                       (long long)ctx->near_cap, (long long)ctx->opt.leaf_cap, ctx->T32, ctx->NT32, ctx->T64,
                       ctx->NT64, ctx->grid32, ctx->grid64, ctx->grid64c, ctx->opt.recheck_pairs,
-                      ctx->pairs_fit ? 1 : 0, use_tc ? ctx->T_tc : 0, use_tc ? ctx->grid_tc : 0);
+                      ctx->pairs_fit ? 1 : 0, use_tc ? ctx->T_tc : 0, use_tc ? ctx->grid_tc : 0,
+                      ctx->small_levels ? 1 : 0);
         if (!ctx->count_graph || ctx->count_graph_key != key) {
             if (ctx->count_graph) cudaGraphExecDestroy(ctx->count_graph);
             ctx->count_graph = nullptr;
@@ -2103,12 +2116,12 @@ int slr_count(slr_ctx *ctx, int D, slr_result *out) { return count_levels(ctx, D
 // ---- checkpoint / resume ----------------------------------------------------
 namespace {
 constexpr uint32_t kCkptMagic = 0x43524c53u;   // "SLRC"
-constexpr uint32_t kCkptVersion = 3;
+constexpr uint32_t kCkptVersion = 4;
 
 // The FP32 tile (boxes and threads per CTA) is part of the state: small tiles
 // split a product's inputs over lanes, so the summation order, and with it
 // which boxes land on the FP64 re-check list, depends on the tile.  A resume
-// runs the checkpoint's tile whatever the autotuner of its context chose.
+// runs the checkpoint's tiles whatever the autotuner of its context chose.
 struct CkptHeader {
     uint32_t magic, version;
     int32_t D, t;
@@ -2116,7 +2129,9 @@ struct CkptHeader {
     uint64_t n_codes;
     uint64_t counters_bytes;
     int32_t tile_boxes, tile_threads;
+    int32_t small_levels, reserved;   // level_tile's rule; not in version 3, whose counts all used it
 };
+constexpr size_t kCkptHeader3 = offsetof(CkptHeader, small_levels);
 
 uint64_t fnv1a(uint64_t h, const void *p, size_t n) {
     const unsigned char *c = static_cast<const unsigned char *>(p);
@@ -2175,7 +2190,7 @@ int slr_count_checkpoint(slr_ctx *ctx, int D, int t, void *buf, size_t cap, size
     if (!buf || cap < need)
         return fail(ctx, SLR_EINVAL, "the checkpoint needs %zu bytes (buffer of %zu)", need, buf ? cap : (size_t)0);
     CkptHeader h{kCkptMagic, kCkptVersion, D, t, problem_fingerprint(ctx), n, sizeof(slr::LevelCounters),
-                 ctx->T32, ctx->NT32};
+                 ctx->T32, ctx->NT32, ctx->small_levels ? 1 : 0, 0};
     unsigned char *p = static_cast<unsigned char *>(buf);
     std::memcpy(p, &h, sizeof h);
     std::memcpy(p + sizeof h, ctx->h_ctr, sizeof(slr::LevelCounters));
@@ -2192,12 +2207,15 @@ int slr_count_resume(slr_ctx *ctx, const void *buf, size_t bytes, slr_result *ou
     int rc = check_ready(ctx);
     if (rc) return rc;
     if ((rc = check_resumable(ctx, "slr_count_resume"))) return rc;
-    const size_t head = sizeof(CkptHeader) + sizeof(slr::LevelCounters);
-    if (!buf || bytes < head) return fail(ctx, SLR_EINVAL, "not a checkpoint (%zu bytes)", bytes);
+    if (!buf || bytes < sizeof(CkptHeader)) return fail(ctx, SLR_EINVAL, "not a checkpoint (%zu bytes)", bytes);
     const unsigned char *p = static_cast<const unsigned char *>(buf);
     CkptHeader h;
     std::memcpy(&h, p, sizeof h);
-    if (h.magic != kCkptMagic || h.version != kCkptVersion || h.counters_bytes != sizeof(slr::LevelCounters))
+    if (h.version == 3) h.small_levels = 1;
+    const size_t hsize = h.version == 3 ? kCkptHeader3 : sizeof h, head = hsize + sizeof(slr::LevelCounters);
+    if (bytes < head) return fail(ctx, SLR_EINVAL, "not a checkpoint (%zu bytes)", bytes);
+    if (h.magic != kCkptMagic || (h.version != kCkptVersion && h.version != 3) ||
+        h.counters_bytes != sizeof(slr::LevelCounters))
         return fail(ctx, SLR_EINVAL, "not a checkpoint of this library version");
     if (h.D < 1 || h.D > slr::kMaxDepth || h.t < 0 || h.t >= h.D)
         return fail(ctx, SLR_EINVAL, "checkpoint with D=%d, t=%d is not valid", h.D, h.t);
@@ -2209,33 +2227,36 @@ int slr_count_resume(slr_ctx *ctx, const void *buf, size_t bytes, slr_result *ou
     if (h.fingerprint != problem_fingerprint(ctx))
         return fail(ctx, SLR_EINVAL, "the checkpoint is of another network, box, property or result options");
     std::vector<unsigned char> ctr(sizeof(slr::LevelCounters));
-    std::memcpy(ctr.data(), p + sizeof h, ctr.size());
+    std::memcpy(ctr.data(), p + hsize, ctr.size());
     const slr::LevelCounters *c = reinterpret_cast<const slr::LevelCounters *>(ctr.data());
     if (c->frontier_n[h.t + 1] != h.n_codes)
         return fail(ctx, SLR_EINVAL, "checkpoint counters and frontier disagree");
     std::vector<uint64_t> codes((size_t)h.n_codes);
     if (h.n_codes > 0) std::memcpy(codes.data(), p + head, (size_t)h.n_codes * sizeof(uint64_t));
     ResumeState rs{h.t + 1, c, codes.data(), (int64_t)h.n_codes};
-    if (ctx->wide || (h.tile_boxes == ctx->T32 && h.tile_threads == ctx->NT32))
-        return count_levels(ctx, h.D, out, h.D, &rs);
-    // the checkpoint's FP32 tile for the resumed levels, the context's own afterwards
-    TileChoice tile{};
-    for (const TileChoice &cand : tile_candidates(ctx->nf))
-        if (cand.T == h.tile_boxes && cand.NT == h.tile_threads) tile = cand;
-    if (tile.T == 0)
-        return fail(ctx, SLR_EINVAL, "the checkpoint's tile %d x %d is not available for this network", h.tile_boxes,
-                    h.tile_threads);
-    const int T0 = ctx->T32, NT0 = ctx->NT32, g0 = ctx->grid32;
-    const size_t s0 = ctx->smem32;
-    ctx->T32 = tile.T;
-    ctx->NT32 = tile.NT;
-    ctx->smem32 = tile.smem;
-    ctx->grid32 = tile.blocks * ctx->sm_count;
+    if (ctx->wide) return count_levels(ctx, h.D, out, h.D, &rs);
+    // the checkpoint's FP32 tiles for the resumed levels, the context's own afterwards
+    const TileChoice own = context_tile(ctx);
+    TileChoice tile = own;
+    if (h.tile_boxes != own.T || h.tile_threads != own.NT) {
+        tile.T = 0;
+        for (const TileChoice &cand : tile_candidates(ctx->nf))
+            if (cand.T == h.tile_boxes && cand.NT == h.tile_threads) tile = cand;
+        if (tile.T == 0)
+            return fail(ctx, SLR_EINVAL, "the checkpoint's tile %d x %d is not available for this network",
+                        h.tile_boxes, h.tile_threads);
+    }
+    auto set = [&](const TileChoice &c, bool small_levels) {
+        ctx->T32 = c.T;
+        ctx->NT32 = c.NT;
+        ctx->smem32 = c.smem;
+        ctx->grid32 = c.blocks * ctx->sm_count;
+        ctx->small_levels = small_levels;
+    };
+    const bool own_small = ctx->small_levels;
+    set(tile, h.small_levels != 0);
     rc = count_levels(ctx, h.D, out, h.D, &rs);
-    ctx->T32 = T0;
-    ctx->NT32 = NT0;
-    ctx->grid32 = g0;
-    ctx->smem32 = s0;
+    set(own, own_small);
     return rc;
 }
 
@@ -2479,7 +2500,7 @@ int slr_bounds(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi
         const int grid = (int)std::min<int64_t>(tiles, ctx->grid_tc);
         CK(ctx, slr::launch_eval_tc(ctx->T_tc, grid, ctx->smem_tc, ctx->stream, ctx->nf, ctx->tcp, src, o, 0));
     } else {
-        const TileChoice tile = few_tile(ctx, n);
+        const TileChoice tile = context_tile(ctx);
         const int grid = (int)std::min<int64_t>((n + tile.T - 1) / tile.T, (int64_t)tile.blocks * ctx->sm_count);
         CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, grid, tile.smem, ctx->stream, ctx->nf, src, o, 0));
     }
@@ -2846,8 +2867,6 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
             int p0, p1, T, grid;
             size_t smem;
             slr::BatchShape sh;
-            int T4, grid4;      // the 4-box tile of the same shapes (first steps)
-            size_t smem4;
         };
         std::vector<Group> groups;
         bs->tile_of.assign(P, 0);
@@ -2862,7 +2881,7 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
                 sh.R = std::max(sh.R, n32[j].R);
                 ++j;
             }
-            Group gr{i, j, 0, 0, 0, sh, 0, 0, 0};
+            Group gr{i, j, 0, 0, 0, sh};
             // the group's combined shape may need a smaller tile than each member alone
             for (int tt : kBatchTiles) {
                 if (tt > t) continue;
@@ -2876,9 +2895,6 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
                 break;
             }
             if (!gr.T) return fail(ctx, SLR_EUNSUPPORTED, "a problem of the batch is too large for the fused kernel");
-            gr.T4 = 4;
-            gr.smem4 = slr::eval_smem_bytes<float>(4, sh.d, sh.R, sh.nmp, sh.n_in_max);
-            gr.grid4 = slr::eval_batch_blocks_per_sm_f32(4, gr.smem4) * ctx->sm_count;
             for (int k = i; k < j; ++k) bs->tile_of[k] = gr.T;
             groups.push_back(gr);
             i = j;
@@ -2999,14 +3015,10 @@ int count_batch_sorted(slr_ctx *ctx, int n, const slr_problem *problems, slr_res
                 cudaStream_t st = gi == 0 ? ctx->stream : branch[gi - 1];
                 if (gi > 0) ce = cudaStreamWaitEvent(st, fork, 0);
                 long long *pg = pm + gr.p0 + gi;
-                // few boxes (at most 2^t per problem): 4-box tiles, as few_tile
-                const bool few = gr.grid4 > 0 && t < 20 && ((int64_t)(gr.p1 - gr.p0) << t) <= 4 * (int64_t)ctx->sm_count;
-                const int gT = few ? gr.T4 : gr.T;
-                if (ce == cudaSuccess) ce = slr::launch_tile_prefix(s_m + gr.p0, gr.p1 - gr.p0, gT, pg, st);
+                if (ce == cudaSuccess) ce = slr::launch_tile_prefix(s_m + gr.p0, gr.p1 - gr.p0, gr.T, pg, st);
                 if (ce == cudaSuccess)
-                    ce = slr::launch_eval_batch_f32(gT, few ? gr.grid4 : gr.grid, few ? gr.smem4 : gr.smem, st,
-                                                    dn32 + gr.p0, s_m + gr.p0, o_m + gr.p0, gr.p1 - gr.p0, pg, gr.sh,
-                                                    0);
+                    ce = slr::launch_eval_batch_f32(gr.T, gr.grid, gr.smem, st, dn32 + gr.p0, s_m + gr.p0,
+                                                    o_m + gr.p0, gr.p1 - gr.p0, pg, gr.sh, 0);
                 if (gi > 0 && ce == cudaSuccess) ce = cudaEventRecord(join[gi - 1], st);
                 L += 2;
             }
@@ -3364,7 +3376,7 @@ int eval_by_position(slr_ctx *ctx, slr::BoxSource src, const float *alpha, float
         int64_t launches = 0;
         return n > 0 ? run_wide(ctx, src, n, o, &launches) : SLR_OK;
     }
-    const TileChoice tile = few_tile(ctx, n_hint);
+    const TileChoice tile = context_tile(ctx);
     const int64_t tiles = (n_hint + tile.T - 1) / tile.T;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)tile.blocks * ctx->sm_count));
     CK(ctx, slr::launch_eval_f32(tile.T, tile.NT, grid, tile.smem, ctx->stream, ctx->nf, src, o, 0));

@@ -249,7 +249,7 @@ compact_kernel(const uint64_t *__restrict__ codes_in, const uint8_t *__restrict_
 // one launch instead of two, ranks carried from one run of 1024 boxes to the
 // next.  A level of few boxes is bound by its launches: with one kernel for
 // the compaction (10.0 -> 6.2 us a level, both measured with an event on each
-// side), one for the re-check and the small tiles of few_tile a 2-8-8-1 count
+// side), one for the re-check and the small tiles of level_tile a 2-8-8-1 count
 // of depth 16 takes 407 us instead of 513.  At 4096 boxes the block makes four
 // rounds, still less than the second launch (10.0 -> 6.4 us).
 __global__ void __launch_bounds__(1024)
