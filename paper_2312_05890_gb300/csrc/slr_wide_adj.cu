@@ -20,10 +20,11 @@
 //
 // Layout as the sound wide path: [box][column][neuron], columns 0..d-1 the
 // coefficients of the normalised inputs and column d the constant, neuron
-// row stride NP.  Row kernels: a block is 128 neurons of one box (blockIdx.y),
-// four neighbouring ones per thread (threadIdx.x; a float4 of every column, 512
-// bytes per warp), with the columns split over 16 slices (threadIdx.y) whose
-// sums are added in slice order.  DRAM bounds them:
+// row stride NP.  Row kernels: a block is 32 V neurons of one box (blockIdx.y),
+// V neighbouring ones per thread (threadIdx.x), V = 4 (a float4 of every column,
+// 512 bytes per warp) or, for few boxes, 1 (row_vec); the columns are split over
+// 16 slices (threadIdx.y) whose sums are added in slice order, so V changes no
+// bit.  DRAM bounds them at many boxes:
 // for 256 boxes of a 784-3x256-10 network the backward one takes 285 us and the
 // forward one 183 us a launch (522 and 228 us with one neuron a thread), each
 // reading the state twice (the second pass needs the first's sums; about 2.1 GB
@@ -45,22 +46,28 @@ __device__ __forceinline__ size_t at(int64_t b, int Q, int c, int NP, int p) {
     return ((size_t)b * Q + c) * NP + p;
 }
 
-constexpr int kA4Rows = 4 * kAX;   // neurons of a row kernel's block
-
-__device__ __forceinline__ void ld4(const float *p, float (&v)[4]) {
-    const float4 t = *reinterpret_cast<const float4 *>(p);
-    v[0] = t.x;
-    v[1] = t.y;
-    v[2] = t.z;
-    v[3] = t.w;
+// V neighbouring values at p.
+template <int V>
+__device__ __forceinline__ void ldn(const float *p, float (&v)[V]) {
+    if constexpr (V == 4) {
+        const float4 t = *reinterpret_cast<const float4 *>(p);
+        v[0] = t.x;
+        v[1] = t.y;
+        v[2] = t.z;
+        v[3] = t.w;
+    } else {
+#pragma unroll
+        for (int u = 0; u < V; ++u) v[u] = p[u];
+    }
 }
-// the first `n` of four values (n >= 4: all; the others lie past the layer's width)
-__device__ __forceinline__ void st4(float *p, const float (&v)[4], int n) {
-    if (n >= 4) {
-        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+// the first `n` of V values (n >= V: all; the others lie past the layer's width)
+template <int V>
+__device__ __forceinline__ void stn(float *p, const float (&v)[V], int n) {
+    if (V == 4 && n >= V) {
+        *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1 % V], v[2 % V], v[3 % V]);
         return;
     }
-    for (int u = 0; u < n; ++u) p[u] = v[u];
+    for (int u = 0; u < V && u < n; ++u) p[u] = v[u];
 }
 
 }  // namespace
@@ -114,40 +121,41 @@ wadj_layer1_kernel(const NetParams<float> net, const float *W0t, int NP, const f
 // Hidden layer `layer`: bias on the constant column (bias non-null), concrete
 // bounds of both equations, the slope, and the relaxed equations (Pc, Pr).
 // sc: the five per-neuron scalars (ll, ul, lu, uu, slope), each nb_cap x NP.
+template <int V>
 __global__ void __launch_bounds__(kAX * kAY)
 wadj_fwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, float *C, const float *R, const float *bias,
                 float *sc, int64_t sstride, float *Pc, float *Pr) {
-    __shared__ float psu[kAY][kA4Rows], psl[kAY][kA4Rows];
-    __shared__ float sp[5][kA4Rows];
+    __shared__ float psu[kAY][V * kAX], psl[kAY][V * kAX];
+    __shared__ float sp[5][V * kAX];
     const NetParams<float> &net = a.net;
     const int d = net.d, Q = d + 1, n = net.n[layer];
     const int lane = threadIdx.x, sl = threadIdx.y;
-    const int pb = blockIdx.x * kA4Rows, p0 = pb + 4 * lane;
+    const int pb = blockIdx.x * (V * kAX), p0 = pb + V * lane;
     const int64_t b = blockIdx.y;
     const bool any = p0 < n;
-    float su[4] = {0.f, 0.f, 0.f, 0.f}, sv[4] = {0.f, 0.f, 0.f, 0.f};
+    float su[V] = {}, sv[V] = {};
     if (any) {
-#pragma unroll 4
+#pragma unroll(V == 4 ? 4 : 8)
         for (int c = sl; c < d; c += kAY) {
-            float cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f};
-            ld4(C + at(b, Q, c, NP, p0), cv);
-            if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+            float cv[V], rv[V] = {};
+            ldn<V>(C + at(b, Q, c, NP, p0), cv);
+            if (R != nullptr) ldn<V>(R + at(b, Q, c, NP, p0), rv);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < V; ++u) {
                 su[u] += fabsf(cv[u] + rv[u]);
                 sv[u] += fabsf(cv[u] - rv[u]);
             }
         }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        psu[sl][4 * lane + u] = su[u];
-        psl[sl][4 * lane + u] = sv[u];
+    for (int u = 0; u < V; ++u) {
+        psu[sl][V * lane + u] = su[u];
+        psl[sl][V * lane + u] = sv[u];
     }
     __syncthreads();
-    // the first four slices: one row per thread
+    // the first V slices: one row per thread
     const int row = sl * kAX + lane, p = pb + row;
-    if (sl < kA4Rows / kAX && p < n) {
+    if (sl < V && p < n) {
         float tu = 0.f, tl = 0.f;
         for (int y = 0; y < kAY; ++y) {
             tu += psu[y][row];
@@ -179,19 +187,19 @@ wadj_fwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, float *C, cons
     }
     __syncthreads();
     if (!any) return;
-    float ll[4], ul[4], lu[4], uu[4], al[4];
-    ld4(&sp[0][4 * lane], ll);
-    ld4(&sp[1][4 * lane], ul);
-    ld4(&sp[2][4 * lane], lu);
-    ld4(&sp[3][4 * lane], uu);
-    ld4(&sp[4][4 * lane], al);
-#pragma unroll 4
+    float ll[V], ul[V], lu[V], uu[V], al[V];
+    ldn<V>(&sp[0][V * lane], ll);
+    ldn<V>(&sp[1][V * lane], ul);
+    ldn<V>(&sp[2][V * lane], lu);
+    ldn<V>(&sp[3][V * lane], uu);
+    ldn<V>(&sp[4][V * lane], al);
+#pragma unroll(V == 4 ? 4 : 8)
     for (int c = sl; c < Q; c += kAY) {
-        float cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f}, oc[4], orr[4];
-        ld4(C + at(b, Q, c, NP, p0), cv);
-        if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+        float cv[V], rv[V] = {}, oc[V], orr[V];
+        ldn<V>(C + at(b, Q, c, NP, p0), cv);
+        if (R != nullptr) ldn<V>(R + at(b, Q, c, NP, p0), rv);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < V; ++k) {
             const float u = cv[k] + rv[k], l = cv[k] - rv[k];
             float uh, lh;
             if (ll[k] >= 0.f) {
@@ -212,8 +220,8 @@ wadj_fwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, float *C, cons
             oc[k] = 0.5f * __fadd_rn(uh, lh);
             orr[k] = 0.5f * __fsub_rn(uh, lh);
         }
-        st4(Pc + at(b, Q, c, NP, p0), oc, n - p0);
-        st4(Pr + at(b, Q, c, NP, p0), orr, n - p0);
+        stn<V>(Pc + at(b, Q, c, NP, p0), oc, n - p0);
+        stn<V>(Pr + at(b, Q, c, NP, p0), orr, n - p0);
     }
 }
 
@@ -282,42 +290,43 @@ wadj_rows_kernel(const AdjArgs a, int64_t pos0, int NP, const float *C, const fl
 // adjoints (gPc, gPr) of the products' inputs to those of the pre-activation
 // equations, written as (gC, gR) = (gU + gL, gU - gL) (gR null at layer 1,
 // where U = L); the slope gradient and its projected-Adam step.
-__global__ void __launch_bounds__(kAX * kAY, 2)
+template <int V>
+__global__ void __launch_bounds__(kAX * kAY, V == 4 ? 2 : 1)
 wadj_bwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, const float *C, const float *R, const float *sc,
                 int64_t sstride, const float *gPc, const float *gPr, float *gC, float *gR) {
-    __shared__ float ps[kAY][kA4Rows], pa[kAY][kA4Rows];
-    __shared__ float sp[8][kA4Rows];
+    __shared__ float ps[kAY][V * kAX], pa[kAY][V * kAX];
+    __shared__ float sp[8][V * kAX];
     const NetParams<float> &net = a.net;
     const int d = net.d, Q = d + 1, n = net.n[layer];
     const int lane = threadIdx.x, sl = threadIdx.y;
-    const int pb = blockIdx.x * kA4Rows, p0 = pb + 4 * lane;
+    const int pb = blockIdx.x * (V * kAX), p0 = pb + V * lane;
     const int64_t b = blockIdx.y;
     const bool any = p0 < n;
-    float gs[4] = {0.f, 0.f, 0.f, 0.f}, ga[4] = {0.f, 0.f, 0.f, 0.f};
+    float gs[V] = {}, ga[V] = {};
     if (any) {
-#pragma unroll 2
+#pragma unroll(V == 4 ? 2 : 8)
         for (int c = sl; c < Q; c += kAY) {
-            float gc[4], gr[4], cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f};
-            ld4(gPc + at(b, Q, c, NP, p0), gc);
-            ld4(gPr + at(b, Q, c, NP, p0), gr);
-            ld4(C + at(b, Q, c, NP, p0), cv);
-            if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+            float gc[V], gr[V], cv[V], rv[V] = {};
+            ldn<V>(gPc + at(b, Q, c, NP, p0), gc);
+            ldn<V>(gPr + at(b, Q, c, NP, p0), gr);
+            ldn<V>(C + at(b, Q, c, NP, p0), cv);
+            if (R != nullptr) ldn<V>(R + at(b, Q, c, NP, p0), rv);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < V; ++u) {
                 gs[u] = fmaf(0.5f * (gc[u] + gr[u]), cv[u] + rv[u], gs[u]);
                 ga[u] = fmaf(0.5f * (gc[u] - gr[u]), cv[u] - rv[u], ga[u]);
             }
         }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        ps[sl][4 * lane + u] = gs[u];
-        pa[sl][4 * lane + u] = ga[u];
+    for (int u = 0; u < V; ++u) {
+        ps[sl][V * lane + u] = gs[u];
+        pa[sl][V * lane + u] = ga[u];
     }
     __syncthreads();
-    // the first four slices: one row per thread
+    // the first V slices: one row per thread
     const int row = sl * kAX + lane, p = pb + row;
-    if (sl < kA4Rows / kAX && p < n) {
+    if (sl < V && p < n) {
         float g_s = 0.f, g_a = 0.f;
         for (int y = 0; y < kAY; ++y) {
             g_s += ps[y][row];
@@ -368,24 +377,24 @@ wadj_bwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, const float *C
     }
     __syncthreads();
     if (!any) return;
-    float kind[4], chord[4], sg[4], du[4], su[4], lw[4], dl[4], sl2[4];
-    ld4(&sp[0][4 * lane], kind);
-    ld4(&sp[1][4 * lane], chord);
-    ld4(&sp[2][4 * lane], sg);
-    ld4(&sp[3][4 * lane], du);
-    ld4(&sp[4][4 * lane], su);
-    ld4(&sp[5][4 * lane], lw);
-    ld4(&sp[6][4 * lane], dl);
-    ld4(&sp[7][4 * lane], sl2);
-#pragma unroll 1
+    float kind[V], chord[V], sg[V], du[V], su[V], lw[V], dl[V], sl2[V];
+    ldn<V>(&sp[0][V * lane], kind);
+    ldn<V>(&sp[1][V * lane], chord);
+    ldn<V>(&sp[2][V * lane], sg);
+    ldn<V>(&sp[3][V * lane], du);
+    ldn<V>(&sp[4][V * lane], su);
+    ldn<V>(&sp[5][V * lane], lw);
+    ldn<V>(&sp[6][V * lane], dl);
+    ldn<V>(&sp[7][V * lane], sl2);
+#pragma unroll(V == 4 ? 1 : 8)
     for (int c = sl; c < Q; c += kAY) {
-        float gc[4], gr[4], cv[4], rv[4] = {0.f, 0.f, 0.f, 0.f}, oc[4], orr[4];
-        ld4(gPc + at(b, Q, c, NP, p0), gc);
-        ld4(gPr + at(b, Q, c, NP, p0), gr);
-        ld4(C + at(b, Q, c, NP, p0), cv);
-        if (R != nullptr) ld4(R + at(b, Q, c, NP, p0), rv);
+        float gc[V], gr[V], cv[V], rv[V] = {}, oc[V], orr[V];
+        ldn<V>(gPc + at(b, Q, c, NP, p0), gc);
+        ldn<V>(gPr + at(b, Q, c, NP, p0), gr);
+        ldn<V>(C + at(b, Q, c, NP, p0), cv);
+        if (R != nullptr) ldn<V>(R + at(b, Q, c, NP, p0), rv);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < V; ++k) {
             const float gu = 0.5f * (gc[k] + gr[k]), gl = 0.5f * (gc[k] - gr[k]);
             float oU, oL;
             if (kind[k] == 0.f) {
@@ -406,8 +415,8 @@ wadj_bwd_kernel(const AdjArgs a, int layer, int64_t pos0, int NP, const float *C
             oc[k] = oU + oL;
             orr[k] = oU - oL;
         }
-        st4(gC + at(b, Q, c, NP, p0), oc, n - p0);
-        if (gR != nullptr) st4(gR + at(b, Q, c, NP, p0), orr, n - p0);
+        stn<V>(gC + at(b, Q, c, NP, p0), oc, n - p0);
+        if (gR != nullptr) stn<V>(gR + at(b, Q, c, NP, p0), orr, n - p0);
     }
 }
 
@@ -489,10 +498,22 @@ cudaError_t launch_wadj_layer1(const NetParams<float> &net, const float *W0t, in
     return cudaGetLastError();
 }
 
+// Neurons a thread of the row kernels takes: four where the blocks of 128 fill
+// the GPU, one where they are few or a layer fills few lanes of one (there the
+// kernels wait for their loads, and one neuron a thread has more blocks and
+// keeps more columns in flight).  784-2x128-5, four / one: 20 boxes 394 / 320 us,
+// 100 boxes 654 / 686 us; 784-3x256-5: one box 509 / 413 us, 50 boxes 1017 / 1050 us.
+// Below 128 inputs a thread has few columns and four is never slower.
+static int row_vec(int d, int n, int nb) {
+    return d >= 128 && (n <= kAX || (int64_t)((n + 4 * kAX - 1) / (4 * kAX)) * nb <= 64) ? 1 : 4;
+}
+
 cudaError_t launch_wadj_fwd(const AdjArgs &a, int layer, int64_t pos0, int nb, int NP, float *C, const float *R,
                             const float *bias, float *sc, int64_t sstride, float *Pc, float *Pr, cudaStream_t s) {
-    wadj_fwd_kernel<<<dim3((a.net.n[layer] + kA4Rows - 1) / kA4Rows, nb), dim3(kAX, kAY), 0, s>>>(
-        a, layer, pos0, NP, C, R, bias, sc, sstride, Pc, Pr);
+    const int n = a.net.n[layer], V = row_vec(a.net.d, n, nb);
+    auto k = V == 4 ? wadj_fwd_kernel<4> : wadj_fwd_kernel<1>;
+    k<<<dim3((n + V * kAX - 1) / (V * kAX), nb), dim3(kAX, kAY), 0, s>>>(a, layer, pos0, NP, C, R, bias, sc, sstride,
+                                                                         Pc, Pr);
     return cudaGetLastError();
 }
 
@@ -505,8 +526,10 @@ cudaError_t launch_wadj_rows(const AdjArgs &a, int64_t pos0, int nb, int NP, con
 cudaError_t launch_wadj_bwd(const AdjArgs &a, int layer, int64_t pos0, int nb, int NP, const float *C, const float *R,
                             const float *sc, int64_t sstride, const float *gPc, const float *gPr, float *gC, float *gR,
                             cudaStream_t s) {
-    wadj_bwd_kernel<<<dim3((a.net.n[layer] + kA4Rows - 1) / kA4Rows, nb), dim3(kAX, kAY), 0, s>>>(
-        a, layer, pos0, NP, C, R, sc, sstride, gPc, gPr, gC, gR);
+    const int n = a.net.n[layer], V = row_vec(a.net.d, n, nb);
+    auto k = V == 4 ? wadj_bwd_kernel<4> : wadj_bwd_kernel<1>;
+    k<<<dim3((n + V * kAX - 1) / (V * kAX), nb), dim3(kAX, kAY), 0, s>>>(a, layer, pos0, NP, C, R, sc, sstride, gPc,
+                                                                         gPr, gC, gR);
     return cudaGetLastError();
 }
 
