@@ -408,8 +408,9 @@ def main():
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
         tf32_peak = peaks["bf16_tflops"] * TF32_PER_BF16
         ach = gemm_flop / (gemm_ms / 1e3) / 1e12
+        product = "wide_layer_kernel" if p.d >= 64 and p.prop.R <= 16 else "wide_gemm_kernel"
         roofline = {"bound": "tensor", "achieved": ach, "peak": tf32_peak, "unit": "TFLOP/s",
-                    "frac": ach / tf32_peak, "traffic": None, "kernel": "wide_layer_kernel (tcgen05 kind::tf32)",
+                    "frac": ach / tf32_peak, "traffic": None, "kernel": f"{product} (tcgen05 kind::tf32)",
                     "peak_basis": f"measured bf16 burst {peaks['bf16_tflops']} TFLOP/s x nominal TF32/BF16 "
                                   f"ratio {TF32_PER_BF16:.3f}",
                     "flop_basis": "2 M K (2d + 1) per box and layer (W C on d columns, |W| R on d + 1); "

@@ -718,10 +718,8 @@ int build_wide(slr_ctx *ctx, const HostLayers<float> &L) {
                                 w0t + (size_t)j * nf.n[1] + p0, std::min(16, nf.n[1] - p0) * sizeof(float));
         }
         for (int k = 1; k < K; ++k) {
-            const int n_in = nf.n[k], n_out = nf.n[k + 1];
-            const int Mpad = (n_out + 127) & ~127, Kpad = ctx->w_Kpad[k];
-            (void)Mpad;
-            fill_pieces(L, k, n_in, n_out, Kpad, ctx->wt_Kpad[k], host.data() + offs[k], host.data() + offs_t[k]);
+            fill_pieces(L, k, nf.n[k], nf.n[k + 1], ctx->w_Kpad[k], ctx->wt_Kpad[k], host.data() + offs[k],
+                        host.data() + offs_t[k]);
         }
         CK(ctx, cudaMalloc(&ctx->wide_img, total));
         CK(ctx, upload(ctx, ctx->wide_img, host.data(), host_total));
@@ -1065,7 +1063,8 @@ int run_wide_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int64_t *launches) {
 }
 
 // The adjoint of `a`: on the wide path by per-layer products (no weight
-// gradients there), else the one-box-per-CTA kernel.
+// gradients there), else with a warp per box where the network fits that form,
+// else the block kernel.
 int run_adjoint(slr_ctx *ctx, const slr::AdjArgs &a, int grid, int64_t *launches) {
     bool weights = false;
     for (int k = 0; k < ctx->nf.K; ++k) weights = weights || a.dW[k] != nullptr || a.db[k] != nullptr;
@@ -1376,7 +1375,6 @@ int ensure_count_buffers(slr_ctx *ctx) {
         CK(ctx, cudaMalloc(&ctx->cls, (size_t)cap));
         ctx->near_cap = std::max<int64_t>(1024, cap / 4);
         CK(ctx, cudaMalloc(&ctx->near_list, (size_t)ctx->near_cap * sizeof(int64_t)));
-        CK(ctx, cudaMalloc(&ctx->near_list2, (size_t)ctx->near_cap * sizeof(int64_t)));
         ctx->cap = cap;
     }
     if (!ctx->ctr) {
@@ -1808,6 +1806,8 @@ static int count_levels(slr_ctx *ctx, int D, slr_result *out, int t_last, const 
         CK(ctx, cudaMemsetAsync(ctx->alpha_ctr, 0, 2 * (slr::kMaxDepth + 2) * sizeof(unsigned long long), ctx->stream));
     }
     const bool use_tc = ctx->opt.precision == SLR_PREC_TC_TF32 && ctx->tc_ok;
+    if (use_tc && !ctx->near_list2)   // the boxes that its FP32 re-check leaves to the FP64 one
+        CK(ctx, cudaMalloc(&ctx->near_list2, (size_t)ctx->near_cap * sizeof(int64_t)));
     const int compact_grid = std::max(1, ctx->sm_count * 4);
     const bool prof = ctx->opt.profile != 0;
     const size_t n_prof = prof ? (size_t)(D + 1) * 6 : 0;

@@ -75,7 +75,7 @@ cudaError_t launch_compact_batch(const CompactArgs *args, int P, int t, unsigned
 cudaError_t launch_init_batch(const CompactArgs *args, int P, cudaStream_t s);
 
 // Adjoint of the SLR pass (gradients of a linear loss of the row bounds) and
-// projected Adam on the lower ReLU slopes; one box per CTA.
+// projected Adam on the lower ReLU slopes (launch_adjoint: one or a few boxes per CTA).
 enum { kAlphaDefault = 0, kAlphaFree = 1, kAlphaInit = 2 };
 struct AdjArgs {
     NetParams<float> net;
