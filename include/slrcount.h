@@ -279,7 +279,9 @@ int slr_alpha_width(slr_ctx *ctx, int64_t *H);
  * Gradients are those of the piecewise-smooth bounds: at a kink (a ReLU case
  * or a coefficient sign changing) they are one-sided.  Relax mode NEURIFY
  * only (SLR_EUNSUPPORTED otherwise).  `on_device` as in slr_bounds, for every
- * pointer; float32 atomics make d_W and d_b vary in the last bits run to run. */
+ * pointer; float32 atomics make d_W and d_b vary in the last bits run to run.
+ * A NaN in g_lo or g_hi makes what depends on it NaN.  SLR_ETIMEOUT as for
+ * counts (the outputs are then incomplete). */
 int slr_margin_backward(slr_ctx *ctx, int64_t n, const float *box_lo, const float *box_hi,
                         const float *alpha, const float *g_lo, const float *g_hi,
                         float *row_lo, float *row_hi, float *d_alpha,
