@@ -1119,6 +1119,11 @@ std::vector<TileChoice> recheck_candidates(slr_ctx *ctx, bool pairs) {
     return c64;
 }
 
+// The context's FP32 tile: the one the caller set, or the fastest.
+TileChoice context_tile(const slr_ctx *ctx) {
+    return TileChoice{ctx->T32, ctx->NT32, ctx->grid32 / std::max(1, ctx->sm_count), ctx->smem32};
+}
+
 // SMs of a GB300: a constant, so that a count resumed on a part of one runs the same tiles.
 constexpr int kFewTiles = 152;
 
@@ -1128,12 +1133,9 @@ constexpr int kFewTiles = 152;
 // boxes, so few boxes are done soonest on many small tiles (levels 0 to 8 of a
 // 5-6x50-5 tanh count take 45 us each on 4-box tiles, 78 us on its 20-box one,
 // the whole depth-16 count 3.66 -> 3.22 ms).  A tile decides the last bits of a
-// bound, so the rule takes nothing but the level and the context's tile: a
-// level runs the same tile in every form of the count, and bounds and slope
-// steps, which report no tile, run the context's.
-TileChoice context_tile(const slr_ctx *ctx) {
-    return TileChoice{ctx->T32, ctx->NT32, ctx->grid32 / std::max(1, ctx->sm_count), ctx->smem32};
-}
+// bound, so the rule takes nothing but the level and the context's tile (a
+// level runs the same one in a whole, resumed, sharded or allocation-free count),
+// and bounds and slope steps, which report no tile, run the context's.
 TileChoice level_tile(const slr_ctx *ctx, int t) {
     const int64_t most = (int64_t)1 << std::min(t, 40);
     if (ctx->small_levels)
@@ -2129,7 +2131,7 @@ struct CkptHeader {
     uint64_t n_codes;
     uint64_t counters_bytes;
     int32_t tile_boxes, tile_threads;
-    int32_t small_levels, reserved;   // level_tile's rule; not in version 3, whose counts all used it
+    int32_t small_levels, reserved;   // level_tile's rule; not in version 3, which is read as using it
 };
 constexpr size_t kCkptHeader3 = offsetof(CkptHeader, small_levels);
 
